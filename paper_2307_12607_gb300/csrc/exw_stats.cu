@@ -1,114 +1,333 @@
 // exw_stats.cu -- frame statistics of the decision stage: the motion-variance features Var_x(F_mv), Var_y(F_mv) of
-// the environment vector (Sec. IV-C, Eq. 1) and the colour MSE behind the reward's PSNR (Sec. IV-C, Eq. 3).
+// the environment vector (Sec. IV-C, Eq. 1), and the colour MSE (PSNR) and SSIM of the reward (Sec. IV-C, Eq. 3).
 //
-// Both are FP64 reductions over a fixed grid (kStatBlocks x kStatThreads, independent of the GPU), so the order of
-// every addition is fixed and the result is deterministic.  Each thread reads a grid-strided subsequence
-// (coalesced) and keeps plain FP64 sums -- for the variance, of the count and of x - K, y - K and their squares,
-// with one shift K for the whole frame (a value of the field, so the final subtraction loses little) -- which
-// are added in trees across the warp, the block and, in the last block to finish, the blocks.
+// The sums keep FP64 accuracy without the FP64 pipe, which on this part takes one lane's operation per SM clock (a
+// warp instruction 32 clocks; the FP32 pipe takes 128 lanes): a thread forms each difference and square as a pair of
+// floats (two-difference, fused multiply-add residuals) and adds them with the error-free two-sum, the errors and the
+// small terms in words of their own; every kFoldValues values these are folded into a second set, so the small words
+// stay short sums.  Each rounding left is about 2^-48 of a short partial sum and independent of the others, so over an
+// image they average out below FP64's own last bit; short inputs, where they would not, and differences whose squares
+// would leave float's range go through FP64 value by value, as everything did before.
+//
+// Every grid is a function of the sizes only and every sum has a fixed order: results are deterministic and do not
+// depend on the GPU.  The blocks' partials are added by a one-block kernel launched behind them with programmatic
+// serialisation, so no counter in the workspace has to be cleared first.
 #include "exw_device.cuh"
 #include "exw_internal.h"
 
 namespace exw {
 namespace {
 
-constexpr int kStatBlocks = 256, kStatThreads = 256;
+// One block per SM of a 152-SM part: with 256 blocks (the earlier grid) 104 SMs had two and 48 one.
+constexpr int kStatBlocks = 152, kStatThreads = 512;
+constexpr int kFoldValues = 32;             // values a thread adds to its short sums between two folds
+constexpr size_t kWideValues = 1u << 14;    // inputs shorter than this are summed in FP64 throughout
+constexpr int kSumThreads = 256;            // the kernel that adds the partials
+constexpr int kMaxPartials = 1280;          // doubles in the workspace
 
-struct Moments {  // a block's partial: count, shifted sums of x and y, shifted sums of squares
-    double n, mx, my, vx, vy;
-};
-
-// Workspace: the blocks' partial results, then the arrival counter of the last-block pattern.
 struct StatWs {
-    Moments part[kStatBlocks];
-    unsigned int arrived;
+    double part[kMaxPartials];
+    unsigned int reserved;  // keeps the workspace at its size
 };
 
-// The last block to finish (by an atomic ticket after a fence) sees every partial.
-__device__ __forceinline__ bool last_block(unsigned int *arrived) {
-    __shared__ bool last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(arrived, 1u) == gridDim.x - 1;
-    __syncthreads();
-    return last;
+// ------------------------------------------------------------------------------------------------------------
+// Error-free arithmetic on floats (Knuth's two-sum, Dekker's product by fused multiply-add).
+// ------------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void two_diff(float a, float b, float &h, float &l) {  // a - b = h + l exactly
+    h = __fsub_rn(a, b);
+    const float bv = __fsub_rn(a, h), av = __fadd_rn(h, bv);
+    l = __fadd_rn(__fsub_rn(a, av), __fsub_rn(bv, b));
 }
+
+__device__ __forceinline__ float two_sum(float &s, float x) {  // s += x, returns the error of the addition
+    const float t = __fadd_rn(s, x);
+    const float xv = __fsub_rn(t, s), sv = __fsub_rn(t, xv);
+    const float e = __fadd_rn(__fsub_rn(s, sv), __fsub_rn(x, xv));
+    s = t;
+    return e;
+}
+
+// A sum in words of falling size: s, the errors of its additions c, the rest d.  Adding values one by one leaves c and d
+// to plain additions (short sums); joining two sums is error-free down to d.
+struct Words {
+    float s = 0.0f, c = 0.0f, d = 0.0f;
+    __device__ __forceinline__ void small(float x) { d = __fadd_rn(d, two_sum(c, x)); }
+    __device__ __forceinline__ void join(const Words &o) {
+        small(two_sum(s, o.s));
+        small(o.c);
+        d = __fadd_rn(d, o.d);
+    }
+};
+
+struct LinearSum {  // of h + l: the short sum and the one it is folded into
+    Words near, far;
+    __device__ __forceinline__ void add(float h, float l) {
+        near.c = __fadd_rn(near.c, two_sum(near.s, h));
+        near.d = __fadd_rn(near.d, l);
+    }
+    __device__ __forceinline__ void fold() {
+        far.small(near.d);
+        near.d = 0.0f;
+        far.join(near);
+        near = Words{};
+    }
+};
+
+// Of (h + l)^2 = p + e + q + r + l^2 with p = fl(h h), q = fl(2 h l) and their exact residuals e, r.  Plain additions
+// of e would bias the sum by some 2^-51 of itself, so they are error-free too; each kind of term has a word of its own.
+struct SquareSum {
+    Words near, far;
+    float g = 0.0f, k = 0.0f;
+    __device__ __forceinline__ void add(float h, float l) {
+        const float p = __fmul_rn(h, h), h2 = 2.0f * h, q = __fmul_rn(h2, l);
+        const float r = fmaf(l, l, fmaf(h2, l, -q));
+        near.c = __fadd_rn(near.c, two_sum(near.s, p));
+        k = __fadd_rn(k, __fadd_rn(two_sum(near.d, fmaf(h, h, -p)), r));
+        g = __fadd_rn(g, q);
+    }
+    __device__ __forceinline__ void fold() {
+        far.small(near.d);
+        far.small(g);
+        near.d = k;
+        far.join(near);
+        near = Words{};
+        g = k = 0.0f;
+    }
+};
+
+// Differences whose squares, their residuals and 2^28 squares added up stay inside float's range (zero included); NaN and infinities
+// are not in it.  2^-39: the square's residual, down to 2^-48 of it, is still a multiple of 2^-149.
+__device__ __forceinline__ bool float_range(float h) {
+    const float m = fabsf(h);
+    return m == 0.0f || (m >= 0x1p-39f && m < 0x1p40f);
+}
+
+// d += x - y and q += (x - y)^2 in FP64 (not inlined: the FP64 instructions of the rare values stay off the others'
+// path).
+__device__ __noinline__ void wide_square(float x, float y, double &d, double &q) {
+    const double v = (double)x - (double)y;
+    d += v;
+    q = fma(v, v, q);
+}
+
+constexpr int kStatWarps = kStatThreads / 32;
+static_assert(kStatWarps <= 32, "one lane per warp in the last step");
+
+// Block sum of the threads' words: a warp tree in FP32 (its roundings are independent over the thousands of warps of a
+// grid), then one FP64 tree over the warps' words -- FP64 trees in every warp would take 160 times 32 clocks.  Every
+// lane of warp 0 gets the sum.  sh: kStatWarps words, used by one sum only.  One block barrier.
+__device__ __forceinline__ double block_words(Words v, Words *sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Words x;
+        x.s = __shfl_xor_sync(0xFFFFFFFFu, v.s, o);
+        x.c = __shfl_xor_sync(0xFFFFFFFFu, v.c, o);
+        x.d = __shfl_xor_sync(0xFFFFFFFFu, v.d, o);
+        v.join(x);
+    }
+    if (lane == 0) sh[w] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (w == 0) {
+        const Words x = lane < kStatWarps ? sh[lane] : Words{};
+        t = (double)x.s + ((double)x.c + (double)x.d);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+    }
+    return t;
+}
+
+// Block sum of one double per thread (the values that went through FP64): thread 0 gets it.
+__device__ __noinline__ double block_wide(double v, double *sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    __syncthreads();
+    if (lane == 0) sh[w] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int i = 0; i < kStatWarps; ++i) t += sh[i];
+    return t;
+}
+
+// Sum of n partials, fixed order, by the calling warp (lane i takes i, i + 32, ...).
+__device__ __forceinline__ double warp_sum(const double *p, int n) {
+    double v = 0.0;
+    for (int i = threadIdx.x & 31; i < n; i += 32) v += __ldcg(p + i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
+// N consecutive values in one load where the addresses allow it (16 bytes), else one.
+template <typename CT, int N> struct Pack { CT v[N]; };
+template <typename CT, int N> __device__ __forceinline__ Pack<CT, N> load_pack(const CT *p) {
+    Pack<CT, N> r;
+    if constexpr (N == 1) {
+        r.v[0] = __ldg(p);
+    } else {
+        static_assert(sizeof(r) == 16, "one 16-byte load");
+        const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p));
+        memcpy(&r, &u, 16);
+    }
+    return r;
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// Motion variance
+// ------------------------------------------------------------------------------------------------------------
 
 // Shift of the variance's sums: the first finite vector among the first kShiftScan pixels (0 when there is none);
 // every block finds the same one.  Any value of the field keeps the shifted sums' cancellation small.
 constexpr int kShiftScan = 1024;
 
-__global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *__restrict__ mv, size_t n,
-                                                                   StatWs *ws, double *out) {
-    __shared__ double shift[2];
-    __shared__ double red[5][kStatThreads / 32];
+// Partials: count, sums of x - kx and y - ky, sums of their squares, [5][kStatBlocks].  8 bytes read
+// and about 80 FP32 operations a pixel: 1080p 62 us with nine FP64 operations a pixel, 20.8 us now (events around
+// both launches; 2.4 us of reads at the copy rate, the rest launches, tails and issue).
+template <int N>
+__global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *__restrict__ mv, size_t n, bool wide,
+                                                                   double *__restrict__ part) {
+    __shared__ float shift[2];
+    __shared__ Words shp[4][kStatWarps];
+    __shared__ double shw[32];
+    grid_dependency_wait();
+    grid_dependents_launch();  // the kernel that adds the partials
+    constexpr int U = N == 1 ? 8 : 16 / N;  // packs in flight per plane
+    const size_t npack = n / N, stride = (size_t)kStatBlocks * kStatThreads;
+    const size_t first_pack = (size_t)blockIdx.x * kStatThreads + threadIdx.x;
+    Pack<float, N> px[U], py[U];
+    auto fetch = [&](size_t at) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const size_t j = at + u * stride;
+            if (j < npack) {
+                px[u] = load_pack<float, N>(mv + j * N);
+                py[u] = load_pack<float, N>(mv + n + j * N);
+            }
+        }
+    };
+    fetch(first_pack);  // the first values are on their way while the shift is found
     if (threadIdx.x < 32) {
         int first = kShiftScan;
         for (int i0 = 0; i0 < kShiftScan && (size_t)i0 < n && first == kShiftScan; i0 += 32) {
-            const int i = i0 + (int)threadIdx.x;
-            const bool ok = (size_t)i < n && isfinite(__ldg(mv + i)) && isfinite(__ldg(mv + n + i));
-            const unsigned int b = __ballot_sync(0xFFFFFFFFu, ok);
-            if (b) first = i0 + __ffs(b) - 1;
+            const int k = i0 + (int)threadIdx.x;
+            const float x = (size_t)k < n ? __ldg(mv + k) : __int_as_float(0x7FC00000);
+            const float y = (size_t)k < n ? __ldg(mv + n + k) : __int_as_float(0x7FC00000);
+            const unsigned int b = __ballot_sync(0xFFFFFFFFu, isfinite(x) && isfinite(y));
+            if (b) {
+                const int src = __ffs(b) - 1;
+                first = i0 + src;
+                const float sx = __shfl_sync(0xFFFFFFFFu, x, src), sy = __shfl_sync(0xFFFFFFFFu, y, src);
+                if (threadIdx.x == 0) {
+                    shift[0] = sx;
+                    shift[1] = sy;
+                }
+            }
         }
-        if (threadIdx.x == 0) {
-            shift[0] = first < kShiftScan ? (double)mv[first] : 0.0;
-            shift[1] = first < kShiftScan ? (double)mv[n + first] : 0.0;
-        }
+        if (threadIdx.x == 0 && first == kShiftScan) shift[0] = shift[1] = 0.0f;
     }
     __syncthreads();
-    const double kx = shift[0], ky = shift[1];
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // count, sums of (x - kx), (y - ky) and of their squares
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const float x = __ldg(mv + i), y = __ldg(mv + n + i);
-        if (!isfinite(x) || !isfinite(y)) continue;
-        const double dx = (double)x - kx, dy = (double)y - ky;
-        v[0] += 1.0;
-        v[1] += dx;
-        v[2] += dy;
-        v[3] = fma(dx, dx, v[3]);
-        v[4] = fma(dy, dy, v[4]);
-    }
-    // plain sums from here on: warp tree, block, then the blocks in a tree in the last block
+    const float kx = shift[0], ky = shift[1];
+    unsigned int cnt = 0u;
+    bool any_rare = false;
+    LinearSum sx, sy;                       // sums of (x - kx), (y - ky)
+    SquareSum qx, qy;                       // and of their squares
+    double r[4] = {0.0, 0.0, 0.0, 0.0};     // the same over the values that go through FP64
+    // One vector: counted, added as pairs, or left for FP64 (true).
+    auto take = [&](float x, float y) -> bool {
+        const bool ok = isfinite(x) && isfinite(y);
+        cnt += ok ? 1u : 0u;
+        float hx, lx, hy, ly;
+        two_diff(x, kx, hx, lx);
+        two_diff(y, ky, hy, ly);
+        const bool in = wide && float_range(hx) && float_range(hy), use = ok && in;
+        hx = use ? hx : 0.0f;
+        lx = use ? lx : 0.0f;
+        hy = use ? hy : 0.0f;
+        ly = use ? ly : 0.0f;
+        sx.add(hx, lx);
+        sy.add(hy, ly);
+        qx.add(hx, lx);
+        qy.add(hy, ly);
+        return ok && !in;
+    };
+    auto take_rare = [&](float x, float y) {
+        wide_square(x, kx, r[0], r[2]);
+        wide_square(y, ky, r[1], r[3]);
+    };
+    static_assert(kFoldValues % (U * N) == 0, "whole rounds between folds");
+    int round = 1;
+    for (size_t i = first_pack; i < npack; ++round) {
+        unsigned int rare = 0u;
 #pragma unroll
-    for (int c = 0; c < 5; ++c) {
+        for (int u = 0; u < U; ++u) {
+            if (i + u * stride >= npack) break;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_xor_sync(0xFFFFFFFFu, v[c], o);
-        if ((threadIdx.x & 31) == 0) red[c][threadIdx.x >> 5] = v[c];
+            for (int j = 0; j < N; ++j) rare |= take(px[u].v[j], py[u].v[j]) ? 1u << (u * N + j) : 0u;
+        }
+        if (rare != 0u) {
+            any_rare = true;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    if (rare & (1u << (u * N + j))) take_rare(px[u].v[j], py[u].v[j]);
+        }
+        if (round % (kFoldValues / (U * N)) == 0) {
+            sx.fold();
+            sy.fold();
+            qx.fold();
+            qy.fold();
+        }
+        i += U * stride;
+        fetch(i);
     }
+    const size_t tail = npack * N + first_pack;  // fewer than N values are left
+    if (tail < n) {
+        const float x = __ldg(mv + tail), y = __ldg(mv + n + tail);
+        if (take(x, y)) {
+            any_rare = true;
+            take_rare(x, y);
+        }
+    }
+    sx.fold();
+    sy.fold();
+    qx.fold();
+    qy.fold();
+    double t[4] = {block_words(sx.far, shp[0]), block_words(sy.far, shp[1]), block_words(qx.far, shp[2]),
+                   block_words(qy.far, shp[3])};
+    if (__syncthreads_or(any_rare ? 1 : 0)) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double w = block_wide(r[c], shw);
+            if (threadIdx.x == 0) t[c] += w;
+        }
+    }
+    cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+    __shared__ unsigned int counts[kStatWarps];
+    if ((threadIdx.x & 31) == 0) counts[threadIdx.x >> 5] = cnt;
     __syncthreads();
     if (threadIdx.x == 0) {
-        Moments &pb = ws->part[blockIdx.x];
-        double t[5];
+        unsigned int c = 0u;  // a block's pixels: at most 2^28 / 152
+        for (int w = 0; w < kStatWarps; ++w) c += counts[w];
+        part[blockIdx.x] = (double)c;
 #pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            t[c] = red[c][0];
-            for (int w = 1; w < kStatThreads / 32; ++w) t[c] += red[c][w];
-        }
-        pb = Moments{t[0], t[1], t[2], t[3], t[4]};
+        for (int k = 0; k < 4; ++k) part[(k + 1) * kStatBlocks + blockIdx.x] = t[k];
     }
-    if (!last_block(&ws->arrived)) return;
-    // the partials of all blocks: thread j takes block j (kStatThreads == kStatBlocks), then a tree
-    static_assert(kStatThreads == kStatBlocks, "one partial per thread");
-    const Moments pj = ws->part[threadIdx.x];
-    double u[5] = {pj.n, pj.mx, pj.my, pj.vx, pj.vy};
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) u[c] += __shfl_xor_sync(0xFFFFFFFFu, u[c], o);
+}
+
+__global__ void __launch_bounds__(kSumThreads) mv_variance_sum_kernel(const double *part, double *out) {
+    __shared__ double t[5];
+    grid_dependency_wait();  // the partials
+    const int w = threadIdx.x >> 5;
+    if (w < 5) {
+        const double v = warp_sum(part + w * kStatBlocks, kStatBlocks);
+        if ((threadIdx.x & 31) == 0) t[w] = v;
     }
-    __syncthreads();  // red is reused
-#pragma unroll
-    for (int c = 0; c < 5; ++c)
-        if ((threadIdx.x & 31) == 0) red[c][threadIdx.x >> 5] = u[c];
     __syncthreads();
     if (threadIdx.x != 0) return;
-    double t[5];
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-        t[c] = red[c][0];
-        for (int w = 1; w < kStatThreads / 32; ++w) t[c] += red[c][w];
-    }
     const double cnt = t[0];
     out[0] = cnt;
     if (cnt == 0.0) {
@@ -118,36 +337,86 @@ __global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *
         out[1] = fmax(t[3] / cnt - ax * ax, 0.0);
         out[2] = fmax(t[4] / cnt - ay * ay, 0.0);
     }
-    ws->arrived = 0u;
 }
 
-template <typename CT>
+// ------------------------------------------------------------------------------------------------------------
+// Colour MSE
+// ------------------------------------------------------------------------------------------------------------
+
+// 2c bytes read a pixel and about 30 FP32 operations a value: 1080p FP32 79 us with four FP64 operations a value,
+// 20.6 us now (events around both launches; 7.3 us of reads at the copy rate).
+template <typename CT, int N>
 __global__ void __launch_bounds__(kStatThreads) color_mse_kernel(const CT *__restrict__ a, const CT *__restrict__ b,
-                                                                 size_t n, StatWs *ws, double *out, bool psnr) {
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    double s = 0.0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const double d = (double)to_f<CT>(a[i]) - (double)to_f<CT>(b[i]);
-        s = fma(d, d, s);
-    }
+                                                                 size_t n, bool wide, double *__restrict__ part) {
+    __shared__ Words shp[kStatWarps];
+    __shared__ double shw[32];
+    grid_dependency_wait();
+    grid_dependents_launch();  // the kernel that adds the partials
+    constexpr int U = N == 1 ? 8 : 16 / N;  // packs in flight per image
+    const size_t npack = n / N, stride = (size_t)kStatBlocks * kStatThreads;
+    const size_t first_pack = (size_t)blockIdx.x * kStatThreads + threadIdx.x;
+    SquareSum q;
+    double r = 0.0, unused = 0.0;
+    bool any_rare = false;
+    auto take = [&](CT va, CT vb) -> bool {
+        float h, l;
+        two_diff(to_f<CT>(va), to_f<CT>(vb), h, l);
+        const bool in = wide && float_range(h);
+        q.add(in ? h : 0.0f, in ? l : 0.0f);
+        return !in;
+    };
+    static_assert(kFoldValues % (U * N) == 0, "whole rounds between folds");
+    int round = 1;
+    for (size_t i = first_pack; i < npack; i += U * stride, ++round) {
+        Pack<CT, N> pa[U], pb[U];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    __shared__ double warps[kStatThreads / 32];
-    if ((threadIdx.x & 31) == 0) warps[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kStatThreads / 32; ++w) t += warps[w];
-        ws->part[blockIdx.x].n = t;
+        for (int u = 0; u < U; ++u) {
+            const size_t j = i + u * stride;
+            if (j < npack) {
+                pa[u] = load_pack<CT, N>(a + j * N);
+                pb[u] = load_pack<CT, N>(b + j * N);
+            }
+        }
+        unsigned int rare = 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i + u * stride >= npack) break;
+#pragma unroll
+            for (int j = 0; j < N; ++j) rare |= take(pa[u].v[j], pb[u].v[j]) ? 1u << (u * N + j) : 0u;
+        }
+        if (rare != 0u) {
+            any_rare = true;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    if (rare & (1u << (u * N + j)))
+                        wide_square(to_f<CT>(pa[u].v[j]), to_f<CT>(pb[u].v[j]), unused, r);
+        }
+        if (round % (kFoldValues / (U * N)) == 0) q.fold();
     }
-    if (!last_block(&ws->arrived) || threadIdx.x != 0) return;
-    double t = 0.0;
-    for (int k = 0; k < (int)gridDim.x; ++k) t += ws->part[k].n;
-    const double mse = t / (double)n;
+    const size_t tail = npack * N + first_pack;  // fewer than N values are left
+    if (tail < n && take(a[tail], b[tail])) {
+        any_rare = true;
+        wide_square(to_f<CT>(a[tail]), to_f<CT>(b[tail]), unused, r);
+    }
+    q.fold();
+    double t = block_words(q.far, shp);
+    if (__syncthreads_or(any_rare ? 1 : 0)) {
+        const double w = block_wide(r, shw);
+        if (threadIdx.x == 0) t += w;
+    }
+    if (threadIdx.x == 0) part[blockIdx.x] = t;
+}
+
+__global__ void __launch_bounds__(32) color_mse_sum_kernel(const double *part, double n, double *out, bool psnr) {
+    grid_dependency_wait();  // the partials
+    const double t = warp_sum(part, kStatBlocks);
+    if (threadIdx.x != 0) return;
+    const double mse = t / n;
     out[0] = mse;
     // PSNR of colours in [0, 1] scaled by 255: 10 log10(255^2 / MSE) = -10 log10(MSE); +inf for equal images
     if (psnr) out[1] = mse == 0.0 ? __longlong_as_double(0x7FF0000000000000ll) : -10.0 * log10(mse);
-    ws->arrived = 0u;
 }
 
 // SSIM (Sec. IV-C, Eq. 3; the standard 11 x 11 Gaussian-window index, sigma 1.5, C1 = 1e-4, C2 = 9e-4 for
@@ -155,16 +424,18 @@ __global__ void __launch_bounds__(kStatThreads) color_mse_kernel(const CT *__res
 // shared memory), filters the five maps a, b, a^2, b^2, ab horizontally into shared memory, then vertically per
 // output, in FP32 on values shifted by -1/2 (variances and covariance are shift-invariant; the shift keeps the
 // raw second moments small), and sums the per-position SSIM in FP64 in a fixed order.
-constexpr int kSsimTile = 32, kSsimIn = kSsimTile + 10;
+constexpr int kSsimTile = 32, kSsimIn = kSsimTile + 10, kSsimBlocks = 256, kSsimThreads = 256;
 
 template <typename CT>
-__global__ void __launch_bounds__(kStatThreads) ssim_kernel(const CT *__restrict__ a, const CT *__restrict__ b,
-                                                            int W, int H, StatWs *ws, double *out) {
+__global__ void __launch_bounds__(kSsimThreads) ssim_kernel(const CT *__restrict__ a, const CT *__restrict__ b,
+                                                            int W, int H, double *__restrict__ part) {
     __shared__ float ia[kSsimIn][kSsimIn + 1], ib[kSsimIn][kSsimIn + 1];
     __shared__ float hor[5][kSsimIn][kSsimTile];
     __shared__ float g[11];
-    __shared__ double red[kStatThreads / 32];
+    __shared__ double red[kSsimThreads / 32];
     const int tid = threadIdx.x;
+    grid_dependency_wait();
+    grid_dependents_launch();  // the kernel that adds the partials
     if (tid < 11) {
         float e[11], sum = 0.0f;
         for (int i = 0; i < 11; ++i) {
@@ -182,7 +453,7 @@ __global__ void __launch_bounds__(kStatThreads) ssim_kernel(const CT *__restrict
         const int X0 = (t % ntx) * kSsimTile, Y0 = (t / ntx) * kSsimTile;
         for (int c = 0; c < 3; ++c) {
             __syncthreads();  // the previous channel's tiles are consumed
-            for (int i = tid; i < kSsimIn * kSsimIn; i += kStatThreads) {
+            for (int i = tid; i < kSsimIn * kSsimIn; i += kSsimThreads) {
                 const int r = i / kSsimIn, q = i - r * kSsimIn, x = X0 + q, y = Y0 + r;
                 const bool in = x < W && y < H;
                 const size_t o = c * plane + (size_t)y * W + x;
@@ -190,7 +461,7 @@ __global__ void __launch_bounds__(kStatThreads) ssim_kernel(const CT *__restrict
                 ib[r][q] = in ? to_f<CT>(b[o]) - 0.5f : 0.0f;
             }
             __syncthreads();
-            for (int i = tid; i < kSsimIn * kSsimTile; i += kStatThreads) {
+            for (int i = tid; i < kSsimIn * kSsimTile; i += kSsimThreads) {
                 const int r = i / kSsimTile, q = i - r * kSsimTile;
                 float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
 #pragma unroll
@@ -209,7 +480,7 @@ __global__ void __launch_bounds__(kStatThreads) ssim_kernel(const CT *__restrict
                 hor[4][r][q] = s4;
             }
             __syncthreads();
-            for (int i = tid; i < kSsimTile * kSsimTile; i += kStatThreads) {
+            for (int i = tid; i < kSsimTile * kSsimTile; i += kSsimThreads) {
                 const int r = i / kSsimTile, q = i - r * kSsimTile;
                 if (X0 + q >= OW || Y0 + r >= OH) continue;
                 float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
@@ -233,22 +504,15 @@ __global__ void __launch_bounds__(kStatThreads) ssim_kernel(const CT *__restrict
     __syncthreads();
     if (tid == 0) {
         double s = red[0];
-        for (int w = 1; w < kStatThreads / 32; ++w) s += red[w];
-        ws->part[blockIdx.x].n = s;
+        for (int w = 1; w < kSsimThreads / 32; ++w) s += red[w];
+        part[blockIdx.x] = s;
     }
-    if (!last_block(&ws->arrived)) return;
-    static_assert(kStatThreads == kStatBlocks, "one partial per thread");
-    double u = tid < (int)gridDim.x ? ws->part[tid].n : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xFFFFFFFFu, u, o);
-    __syncthreads();
-    if ((tid & 31) == 0) red[tid >> 5] = u;
-    __syncthreads();
-    if (tid != 0) return;
-    double s = red[0];
-    for (int w = 1; w < kStatThreads / 32; ++w) s += red[w];
-    out[0] = s / (3.0 * (double)OW * (double)OH);
-    ws->arrived = 0u;
+}
+
+__global__ void __launch_bounds__(32) ssim_sum_kernel(const double *part, int nparts, double count, double *out) {
+    grid_dependency_wait();  // the partials
+    const double t = warp_sum(part, nparts);
+    if (threadIdx.x == 0) out[0] = t / count;
 }
 
 }  // namespace
@@ -256,50 +520,73 @@ __global__ void __launch_bounds__(kStatThreads) ssim_kernel(const CT *__restrict
 size_t stats_workspace_bytes() { return (sizeof(StatWs) + 255) & ~(size_t)255; }
 
 cudaError_t launch_mv_variance(const float *mv, int W, int H, double *out, void *ws, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(&static_cast<StatWs *>(ws)->arrived, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return e;
+    static_assert(5 * kStatBlocks <= kMaxPartials, "the partials fit the workspace");
+    double *const part = static_cast<StatWs *>(ws)->part;
+    const size_t n = (size_t)W * H;
+    const bool vec = ((uintptr_t)mv & 15u) == 0 && (n & 3u) == 0;  // both planes start on 16 bytes
     timing_begin("exw_mv_variance", s);
-    mv_variance_kernel<<<kStatBlocks, kStatThreads, 0, s>>>(mv, (size_t)W * H, static_cast<StatWs *>(ws), out);
+    const bool wide = n >= kWideValues;
+    cudaError_t e = launch_dependent(vec ? mv_variance_kernel<4> : mv_variance_kernel<1>, dim3(kStatBlocks),
+                                     dim3(kStatThreads), 0, s, mv, n, wide, part);
     count_launch();
+    if (e == cudaSuccess) {
+        const double *cpart = part;
+        e = launch_dependent(mv_variance_sum_kernel, dim3(1), dim3(kSumThreads), 0, s, cpart, out);
+        count_launch();
+    }
     timing_end("exw_mv_variance", s);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_color_mse(const void *a, const void *b, exw_dtype cdt, int W, int H, double *out, void *ws,
                              cudaStream_t s, bool psnr) {
-    cudaError_t e = cudaMemsetAsync(&static_cast<StatWs *>(ws)->arrived, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return e;
+    double *const part = static_cast<StatWs *>(ws)->part;
     const size_t n = 3 * (size_t)W * H;
+    const bool vec = (((uintptr_t)a | (uintptr_t)b) & 15u) == 0, wide = n >= kWideValues;
     timing_begin("exw_color_mse", s);
-    if (cdt == EXW_F16)
-        color_mse_kernel<__half><<<kStatBlocks, kStatThreads, 0, s>>>((const __half *)a, (const __half *)b, n,
-                                                                       static_cast<StatWs *>(ws), out, psnr);
-    else
-        color_mse_kernel<float><<<kStatBlocks, kStatThreads, 0, s>>>((const float *)a, (const float *)b, n,
-                                                                      static_cast<StatWs *>(ws), out, psnr);
+    cudaError_t e;
+    if (cdt == EXW_F16) {
+        const __half *x = (const __half *)a, *y = (const __half *)b;
+        e = launch_dependent(vec ? color_mse_kernel<__half, 8> : color_mse_kernel<__half, 1>, dim3(kStatBlocks),
+                             dim3(kStatThreads), 0, s, x, y, n, wide, part);
+    } else {
+        const float *x = (const float *)a, *y = (const float *)b;
+        e = launch_dependent(vec ? color_mse_kernel<float, 4> : color_mse_kernel<float, 1>, dim3(kStatBlocks),
+                             dim3(kStatThreads), 0, s, x, y, n, wide, part);
+    }
     count_launch();
+    if (e == cudaSuccess) {
+        const double *cpart = part;
+        const double dn = (double)n;
+        e = launch_dependent(color_mse_sum_kernel, dim3(1), dim3(32), 0, s, cpart, dn, out, psnr);
+        count_launch();
+    }
     timing_end("exw_color_mse", s);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
-
-}  // namespace exw
-
-namespace exw {
 
 cudaError_t launch_ssim(const void *a, const void *b, exw_dtype cdt, int W, int H, double *out, void *ws,
                         cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(&static_cast<StatWs *>(ws)->arrived, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return e;
+    double *const part = static_cast<StatWs *>(ws)->part;
     timing_begin("exw_ssim", s);
-    if (cdt == EXW_F16)
-        ssim_kernel<__half><<<kStatBlocks, kStatThreads, 0, s>>>((const __half *)a, (const __half *)b, W, H,
-                                                                  static_cast<StatWs *>(ws), out);
-    else
-        ssim_kernel<float><<<kStatBlocks, kStatThreads, 0, s>>>((const float *)a, (const float *)b, W, H,
-                                                                 static_cast<StatWs *>(ws), out);
+    cudaError_t e;
+    if (cdt == EXW_F16) {
+        const __half *x = (const __half *)a, *y = (const __half *)b;
+        e = launch_dependent(ssim_kernel<__half>, dim3(kSsimBlocks), dim3(kSsimThreads), 0, s, x, y, W, H, part);
+    } else {
+        const float *x = (const float *)a, *y = (const float *)b;
+        e = launch_dependent(ssim_kernel<float>, dim3(kSsimBlocks), dim3(kSsimThreads), 0, s, x, y, W, H, part);
+    }
     count_launch();
+    if (e == cudaSuccess) {
+        const double *cpart = part;
+        const int nparts = kSsimBlocks;
+        const double count = 3.0 * (double)(W - 10) * (double)(H - 10);
+        e = launch_dependent(ssim_sum_kernel, dim3(1), dim3(32), 0, s, cpart, nparts, count, out);
+        count_launch();
+    }
     timing_end("exw_ssim", s);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace exw
