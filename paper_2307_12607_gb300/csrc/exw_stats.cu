@@ -419,94 +419,160 @@ __global__ void __launch_bounds__(32) color_mse_sum_kernel(const double *part, d
     if (psnr) out[1] = mse == 0.0 ? __longlong_as_double(0x7FF0000000000000ll) : -10.0 * log10(mse);
 }
 
-// SSIM (Sec. IV-C, Eq. 3; the standard 11 x 11 Gaussian-window index, sigma 1.5, C1 = 1e-4, C2 = 9e-4 for
-// colours in [0, 1]): each block takes 32 x 32 output positions at a time (a 42 x 42 input tile per channel in
-// shared memory), filters the five maps a, b, a^2, b^2, ab horizontally into shared memory, then vertically per
-// output, in FP32 on values shifted by -1/2 (variances and covariance are shift-invariant; the shift keeps the
-// raw second moments small), and sums the per-position SSIM in FP64 in a fixed order.
-constexpr int kSsimTile = 32, kSsimIn = kSsimTile + 10, kSsimBlocks = 256, kSsimThreads = 256;
+// SSIM (Sec. IV-C, Eq. 3; the standard 11 x 11 Gaussian-window index, sigma 1.5, C1 = 1e-4, C2 = 9e-4 for colours in
+// [0, 1]).  A warp takes 64 output columns (two per lane) of one channel and walks down its rows: the next rows' 74
+// columns of both images are loaded two rows ahead into registers and staged in the warp's own shared memory; each
+// lane filters its two columns horizontally from 12 neighbours and adds the result to the 11 outputs whose windows
+// hold the row, which stay in registers (a ring unrolled by 11 rows).  Nothing but the raw rows passes through shared
+// memory.  FP32 on values shifted by -1/2 (variances and covariance are shift-invariant; the shift keeps the raw
+// second moments small); only the sum of the two variances enters the index, so a^2 + b^2 is one map: four maps.
+// The per-position values are added as float pairs, FP64 per warp and beyond.
+//
+// Bound by issue: per output 2 x 44 multiply-adds for the windows, 18 for the products, about 35 for the index.  1080p
+// FP32 136 us with the filtered maps in shared memory (a multiply-add per load, the sum on the FP64 pipe), 55 us now
+// (events around both launches).
+constexpr int kSsimCols = 64, kSsimIn = kSsimCols + 10, kSsimPad = 80;
+constexpr int kSsimWarps = 4, kSsimThreads = 32 * kSsimWarps;
+constexpr int kSsimItems = 12 * 152;  // warps of one wave: 12 per SM of 152 at up to 168 registers
+
+// Rows of outputs per warp, so that a frame gives about one wave of warps; 8 at least (each warp reads 10 rows more).
+struct SsimGrid {
+    int strips, rows, chunks;
+    SsimGrid(int W, int H) {
+        const int OH = H - 10;
+        strips = ceil_div(W - 10, kSsimCols);
+        int c = kSsimItems / (3 * strips);
+        c = c < 1 ? 1 : c > ceil_div(OH, 8) ? ceil_div(OH, 8) : c;
+        rows = ceil_div(OH, c);
+        chunks = ceil_div(OH, rows);
+    }
+    int items() const { return 3 * strips * chunks; }
+    int blocks() const { return ceil_div(items(), kSsimWarps); }
+};
 
 template <typename CT>
-__global__ void __launch_bounds__(kSsimThreads) ssim_kernel(const CT *__restrict__ a, const CT *__restrict__ b,
-                                                            int W, int H, double *__restrict__ part) {
-    __shared__ float ia[kSsimIn][kSsimIn + 1], ib[kSsimIn][kSsimIn + 1];
-    __shared__ float hor[5][kSsimIn][kSsimTile];
-    __shared__ float g[11];
-    __shared__ double red[kSsimThreads / 32];
-    const int tid = threadIdx.x;
+__global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restrict__ a, const CT *__restrict__ b,
+                                                               int W, int H, int strips, int rows, int chunks,
+                                                               double *__restrict__ part) {
+    __shared__ __align__(16) float stage[kSsimWarps][2][2][kSsimPad];  // [warp][row parity][image][column]
+    __shared__ double red[kSsimWarps];
     grid_dependency_wait();
     grid_dependents_launch();  // the kernel that adds the partials
-    if (tid < 11) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int OW = W - 10, OH = H - 10;
+    float g[6];  // the window's weights, symmetric: g[i] = weight i = weight 10 - i
+    {
         float e[11], sum = 0.0f;
         for (int i = 0; i < 11; ++i) {
             e[i] = expf(-(float)((i - 5) * (i - 5)) / 4.5f);
             sum += e[i];
         }
-        g[tid] = e[tid] / sum;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) g[i] = e[i] / sum;
     }
-    const int OW = W - 10, OH = H - 10;
-    const int ntx = (OW + kSsimTile - 1) / kSsimTile, nt = ntx * ((OH + kSsimTile - 1) / kSsimTile);
-    const size_t plane = (size_t)W * H;
     const float C1 = 1e-4f, C2 = 9e-4f;
-    double acc = 0.0;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int X0 = (t % ntx) * kSsimTile, Y0 = (t / ntx) * kSsimTile;
-        for (int c = 0; c < 3; ++c) {
-            __syncthreads();  // the previous channel's tiles are consumed
-            for (int i = tid; i < kSsimIn * kSsimIn; i += kSsimThreads) {
-                const int r = i / kSsimIn, q = i - r * kSsimIn, x = X0 + q, y = Y0 + r;
-                const bool in = x < W && y < H;
-                const size_t o = c * plane + (size_t)y * W + x;
-                ia[r][q] = in ? to_f<CT>(a[o]) - 0.5f : 0.0f;
-                ib[r][q] = in ? to_f<CT>(b[o]) - 0.5f : 0.0f;
-            }
-            __syncthreads();
-            for (int i = tid; i < kSsimIn * kSsimTile; i += kSsimThreads) {
-                const int r = i / kSsimTile, q = i - r * kSsimTile;
-                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
+    double total = 0.0;
+    const int item = blockIdx.x * kSsimWarps + wid;
+    if (item < 3 * strips * chunks) {
+        // a strip's chunks are neighbours, then its channels: warps of a block share rows
+        const int strip = item % strips, rest = item / strips, chunk = rest % chunks, ch = rest / chunks;
+        const int X0 = strip * kSsimCols, Y0 = chunk * rows;
+        const int nrow = min(rows, OH - Y0) + 10;  // input rows
+        const CT *pa = a + (size_t)ch * W * H + (size_t)Y0 * W + X0, *pb = b + (size_t)ch * W * H + (size_t)Y0 * W + X0;
+        const int left = W - X0;  // columns of the frame from X0
+        // this lane's columns of a row: lane, lane + 32, lane + 64 (the last for 10 lanes); outside the frame a value
+        // that no output of the frame uses.  As loaded: converted and shifted when they are staged, two rows later
+        struct Row {
+            CT a[3], b[3];
+        };
+        auto fetch = [&](int r) {
+            Row v;
 #pragma unroll
-                for (int j = 0; j < 11; ++j) {
-                    const float va = ia[r][q + j], vb = ib[r][q + j], w = g[j];
-                    s0 = fmaf(w, va, s0);
-                    s1 = fmaf(w, vb, s1);
-                    s2 = fmaf(w, va * va, s2);
-                    s3 = fmaf(w, vb * vb, s3);
-                    s4 = fmaf(w, va * vb, s4);
+            for (int i = 0; i < 3; ++i) {
+                const int x = lane + 32 * i;
+                const bool in = x < kSsimIn && x < left && r < nrow;
+                const size_t o = (size_t)r * W + x;
+                v.a[i] = in ? __ldg(pa + o) : CT(0.0f);
+                v.b[i] = in ? __ldg(pb + o) : CT(0.0f);
+            }
+            return v;
+        };
+        const bool ok0 = X0 + 2 * lane < OW, ok1 = X0 + 2 * lane + 1 < OW;
+        float acc[11][4][2];  // output row o in slot o mod 11: maps a, b, a^2 + b^2, ab of the lane's two columns
+        LinearSum sum;
+        Row n0 = fetch(0), n1 = fetch(1);
+        for (int base = 0; base < nrow; base += 11) {
+#pragma unroll
+            for (int u = 0; u < 11; ++u) {
+                const int r = base + u;
+                if (r >= nrow) break;
+                float(*st)[kSsimPad] = stage[wid][r & 1];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    if (lane + 32 * i < kSsimPad) {
+                        st[0][lane + 32 * i] = to_f<CT>(n0.a[i]) - 0.5f;
+                        st[1][lane + 32 * i] = to_f<CT>(n0.b[i]) - 0.5f;
+                    }
                 }
-                hor[0][r][q] = s0;
-                hor[1][r][q] = s1;
-                hor[2][r][q] = s2;
-                hor[3][r][q] = s3;
-                hor[4][r][q] = s4;
-            }
-            __syncthreads();
-            for (int i = tid; i < kSsimTile * kSsimTile; i += kSsimThreads) {
-                const int r = i / kSsimTile, q = i - r * kSsimTile;
-                if (X0 + q >= OW || Y0 + r >= OH) continue;
-                float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+                n0 = n1;
+                n1 = fetch(r + 2);
+                __syncwarp();  // the row is staged (the other parity's reads ended before this row's writes began)
+                float va[12], vb[12], h[4][2];
 #pragma unroll
-                for (int k = 0; k < 11; ++k) {
-                    const float w = g[k];
-#pragma unroll
-                    for (int v = 0; v < 5; ++v) m[v] = fmaf(w, hor[v][r + k][q], m[v]);
+                for (int j = 0; j < 6; ++j) {
+                    const float2 x = *reinterpret_cast<const float2 *>(&st[0][2 * lane + 2 * j]);
+                    const float2 y = *reinterpret_cast<const float2 *>(&st[1][2 * lane + 2 * j]);
+                    va[2 * j] = x.x;
+                    va[2 * j + 1] = x.y;
+                    vb[2 * j] = y.x;
+                    vb[2 * j + 1] = y.y;
                 }
-                const float va2 = m[2] - m[0] * m[0], vb2 = m[3] - m[1] * m[1], cab = m[4] - m[0] * m[1];
-                const float mua = m[0] + 0.5f, mub = m[1] + 0.5f;
-                const float num = (2.0f * mua * mub + C1) * (2.0f * cab + C2);
-                const float den = (mua * mua + mub * mub + C1) * (va2 + vb2 + C2);
-                acc += (double)(num / den);
+#pragma unroll
+                for (int j = 0; j < 12; ++j) {
+                    const float x = va[j], y = vb[j], q = fmaf(x, x, y * y), p = x * y;
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {  // column c takes neighbours c .. c + 10
+                        const int i = j - c;
+                        if (i < 0 || i > 10) continue;
+                        const float w = g[i < 6 ? i : 10 - i];
+                        h[0][c] = i == 0 ? w * x : fmaf(w, x, h[0][c]);
+                        h[1][c] = i == 0 ? w * y : fmaf(w, y, h[1][c]);
+                        h[2][c] = i == 0 ? w * q : fmaf(w, q, h[2][c]);
+                        h[3][c] = i == 0 ? w * p : fmaf(w, p, h[3][c]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 11; ++i) {  // row r is window row i of output r - i, in slot (u - i) mod 11
+                    const int slot = (u - i + 11) % 11;
+                    const float w = g[i < 6 ? i : 10 - i];
+#pragma unroll
+                    for (int m = 0; m < 4; ++m)
+#pragma unroll
+                        for (int c = 0; c < 2; ++c)
+                            acc[slot][m][c] = i == 0 ? w * h[m][c] : fmaf(w, h[m][c], acc[slot][m][c]);
+                }
+                if (r >= 10) {  // output row r - 10 is complete
+                    const int slot = (u + 1) % 11;
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const float ma = acc[slot][0][c], mb = acc[slot][1][c];
+                        const float vab = acc[slot][2][c] - ma * ma - mb * mb, cab = acc[slot][3][c] - ma * mb;
+                        const float mua = ma + 0.5f, mub = mb + 0.5f;
+                        const float num = (2.0f * mua * mub + C1) * (2.0f * cab + C2);
+                        const float den = (mua * mua + mub * mub + C1) * (vab + C2);
+                        sum.add(c == 0 ? (ok0 ? num / den : 0.0f) : (ok1 ? num / den : 0.0f), 0.0f);
+                    }
+                }
             }
+            sum.fold();
         }
+        total = (double)sum.far.s + ((double)sum.far.c + (double)sum.far.d);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-    if ((tid & 31) == 0) red[tid >> 5] = acc;
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
+    if (lane == 0) red[wid] = total;
     __syncthreads();
-    if (tid == 0) {
-        double s = red[0];
-        for (int w = 1; w < kSsimThreads / 32; ++w) s += red[w];
-        part[blockIdx.x] = s;
-    }
+    if (threadIdx.x == 0) part[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
 }
 
 __global__ void __launch_bounds__(32) ssim_sum_kernel(const double *part, int nparts, double count, double *out) {
@@ -568,19 +634,22 @@ cudaError_t launch_color_mse(const void *a, const void *b, exw_dtype cdt, int W,
 cudaError_t launch_ssim(const void *a, const void *b, exw_dtype cdt, int W, int H, double *out, void *ws,
                         cudaStream_t s) {
     double *const part = static_cast<StatWs *>(ws)->part;
+    const SsimGrid gr(W, H);
     timing_begin("exw_ssim", s);
     cudaError_t e;
     if (cdt == EXW_F16) {
         const __half *x = (const __half *)a, *y = (const __half *)b;
-        e = launch_dependent(ssim_kernel<__half>, dim3(kSsimBlocks), dim3(kSsimThreads), 0, s, x, y, W, H, part);
+        e = launch_dependent(ssim_kernel<__half>, dim3(gr.blocks()), dim3(kSsimThreads), 0, s, x, y, W, H,
+                             gr.strips, gr.rows, gr.chunks, part);
     } else {
         const float *x = (const float *)a, *y = (const float *)b;
-        e = launch_dependent(ssim_kernel<float>, dim3(kSsimBlocks), dim3(kSsimThreads), 0, s, x, y, W, H, part);
+        e = launch_dependent(ssim_kernel<float>, dim3(gr.blocks()), dim3(kSsimThreads), 0, s, x, y, W, H,
+                             gr.strips, gr.rows, gr.chunks, part);
     }
     count_launch();
     if (e == cudaSuccess) {
         const double *cpart = part;
-        const int nparts = kSsimBlocks;
+        const int nparts = gr.blocks();
         const double count = 3.0 * (double)(W - 10) * (double)(H - 10);
         e = launch_dependent(ssim_sum_kernel, dim3(1), dim3(32), 0, s, cpart, nparts, count, out);
         count_launch();

@@ -105,3 +105,26 @@ def test_non_finite_colours_reach_the_result(b):
     assert b.exw_color_mse(on_gpu(x, 0), on_gpu(y, 0)) == math.inf
     y[1, 40, 45] = np.nan
     assert math.isnan(b.exw_color_mse(on_gpu(x, 0), on_gpu(y, 0)))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float16])
+@pytest.mark.parametrize("W,H", [(11, 11), (12, 19), (74, 18), (75, 21), (138, 97), (139, 40)])
+def test_ssim_strips_and_chunks(b, W, H, dtype):
+    # one output, and the edges of a warp's 64 columns and of its rows.  The bar is that of the oracle test: window
+    # moments within about 1e-7, and an error e in a variance moves a window's SSIM by at most e / C2 (C2 = 9e-4)
+    rng = np.random.default_rng(W + 100 * H)
+    x = rng.uniform(size=(3, H, W)).astype(dtype)
+    y = np.clip(x + rng.normal(scale=0.08, size=x.shape), 0, 1).astype(dtype)
+    g = np.exp(-(np.arange(11) - 5.0) ** 2 / 4.5)
+    g /= g.sum()
+
+    def mean(v):
+        v = sum(g[i] * v[:, :, i:W - 10 + i] for i in range(11))
+        return sum(g[i] * v[:, i:H - 10 + i, :] for i in range(11))
+
+    p, q = x.astype(np.float64), y.astype(np.float64)
+    mp, mq = mean(p), mean(q)
+    vp, vq, c = mean(p * p) - mp * mp, mean(q * q) - mq * mq, mean(p * q) - mp * mq
+    want = (((2 * mp * mq + 1e-4) * (2 * c + 9e-4)) / ((mp * mp + mq * mq + 1e-4) * (vp + vq + 9e-4))).mean()
+    for offset in (0, 1):
+        assert abs(b.exw_ssim(on_gpu(x, offset), on_gpu(y, offset)) - want) <= 2e-4
