@@ -25,6 +25,7 @@
 namespace exw {
 
 cudaError_t launch_engine(const EngineParams &ep, bool fill, int shape, int grid, cudaStream_t s);
+cudaError_t launch_engine_load(const EngineParams &ep, bool fill, int shape, int grid, cudaStream_t s);
 
 constexpr size_t kEngineHeader = 256;  // status word
 
@@ -142,10 +143,16 @@ static bool build_params(EngineParams *ep, const EngineSpec *specs, int first, i
         p.ncoarse = l.ncoarse;
         p.status = ep->status;
         st.cdt = (int)f.cdt;
-        const int a = f.cdt == EXW_F16 ? 8 : 4;  // TMA: rows and bases 16-byte aligned
-        st.tma = sc.tma && fn != nullptr && (f.W % a) == 0 && ((uintptr_t)f.color & 15u) == 0 &&
-                 ((uintptr_t)f.depth & 15u) == 0 && ((uintptr_t)f.mv & 15u) == 0;
-        if (st.tma) {
+        // Windows by TMA where rows and bases are 16-byte aligned; else by the loader warps where every row starts at a
+        // whole word (all float colour, half colour of even width); else, or if the caller asked for it, global-memory
+        // reads.  1918 x 1079 FP32, 8 frames: global 1111 us, loaders 655; 1366 x 768 FP16: 548 and 382; 3838 x 2158
+        // FP16 without fill: 462 and 270.  Half colour of odd width (1917 x 1079) would take 1255 against 1170: its
+        // rows have to be shifted by half a word on the way.
+        const int a = f.cdt == EXW_F16 ? 8 : 4;
+        const bool words = f.cdt == EXW_F32 || ((f.W & 1) == 0 && ((uintptr_t)f.color & 3u) == 0);
+        st.stage = sc.tma && words ? kStageLoad : kStageNone;
+        if (sc.tma && fn != nullptr && (f.W % a) == 0 && ((uintptr_t)f.color & 15u) == 0 &&
+            ((uintptr_t)f.depth & 15u) == 0 && ((uintptr_t)f.mv & 15u) == 0) {
             const int bx = win_x(sc.shape, f.cdt), by = win_y(sc.shape, f.cdt);
             const bool ok =
                 encode(fn, &ep->maps[i][0],
@@ -153,8 +160,9 @@ static bool build_params(EngineParams *ep, const EngineSpec *specs, int first, i
                        f.W, f.H, 3, f.cdt == EXW_F16 ? 2 : 4, bx, by) &&
                 encode(fn, &ep->maps[i][1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, f.depth, f.W, f.H, 1, 4, bx, by) &&
                 encode(fn, &ep->maps[i][2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, f.mv, f.W, f.H, 2, 4, bx, by);
-            if (!ok) st.tma = 0;
+            if (ok) st.stage = kStageTma;
         }
+        ep->loaders |= st.stage == kStageLoad ? 1 : 0;
         st.nregions = ceil_div(f.W, 32) * ceil_div(f.H, 32);
         st.ntiles = l.n5x * l.n5y;
         st.nfix = fill ? (int)kFixupItems : 0;
@@ -209,7 +217,10 @@ static cudaError_t run_all(EngineParams *ep, const EngineSpec *specs, int n, int
                               const_cast<float2 *>(p.tile_depth), const_cast<float4 *>(p.region_bounds), p.fh, s);
             if (e == cudaSuccess) e = launch_plan(p, (exw_dtype)ep->st[i].cdt, sc.shape, s);
         }
-        if (e == cudaSuccess) e = launch_engine(*ep, fill, sc.shape, tiles < sms ? tiles : sms, s);
+        if (e == cudaSuccess) {
+            const int grid = tiles < sms ? tiles : sms;
+            e = ep->loaders ? launch_engine_load(*ep, fill, sc.shape, grid, s) : launch_engine(*ep, fill, sc.shape, grid, s);
+        }
     }
     return e;
 }

@@ -1,5 +1,6 @@
 // exw_engine.cuh -- the forward pass (stages (a0), (a), (b), (c) for P_1..P_3, Sec. IV-B) of any number of frames
-// or streams as ONE warp-specialised persistent kernel: one CTA per SM, 25 warps.
+// or streams as ONE warp-specialised persistent kernel: one CTA per SM, 25 warps (28 with
+// the loaders).
 //
 // Work items of all streams (a stream = one source frame with its outputs) sit in one queue, laid out diagonally --
 // motion-bounds regions of stream d, tile plans of stream d-1, target tiles of stream d-2, fix-ups of stream d-3
@@ -11,6 +12,9 @@
 //                    (cp.async.bulk.tensor, mbarrier completion) and, while they land, writes the tile's plan, its
 //                    splat candidates and the per-fraction constants of uniform tiles, one item ahead of the
 //                    consumers.
+//   3 loader warps:  (LOAD) stage the windows of streams whose rows or bases are not multiples of 16 bytes, which TMA
+//                    cannot read (854 x 480, 1366 x 768, odd widths): asynchronous copies of 8 or 4 bytes, in the same
+//                    slots and layout.  A kernel of its own: in the common one they cost 1 to 2% at aligned sizes.
 //   3 x 8 consumer warps: a bounds item gives each half group one 32 x 32 source region, a plan item each warp one
 //                    target tile, a fix-up item all of them a slice; for a target tile all of them splat (modes
 //                    1-3), then group g computes fraction k0 + g -- each thread a 2 x 2 pixel block -- fills and
@@ -32,7 +36,9 @@ namespace exw {
 constexpr int kGroupThreads = 256;                          // one fraction: 16 x 16 blocks of 2 x 2 pixels
 constexpr int kConsumerThreads = kMaxFrac * kGroupThreads;  // 768
 constexpr int kConsumerWarps = kConsumerThreads / 32;       // 24
-constexpr int kEngineThreads = kConsumerThreads + 32;       // + the producer warp
+constexpr int kLoaderWarps = 3;                             // (registers are allocated to four warps at a time anyway)
+constexpr int kLoaderThreads = 32 * kLoaderWarps;
+template <bool LOAD> constexpr int kEngineThreads = kConsumerThreads + 32 + (LOAD ? kLoaderThreads : 0);  // + the producer warp
 constexpr int kBarConsumers = 1;                            // named barriers: 1 all consumers, 2 + g group g,
 constexpr int kBarBounds = 11;  // 5 + h half group h (bounds), 11 + g group g (bounds)
 constexpr int kMaxStreams = 48;                             // streams per launch (kernel-parameter space)
@@ -57,9 +63,11 @@ constexpr int kSlotEnd = 0, kSlotBounds = 1, kSlotPlans = 2, kSlotTile = 3, kSlo
 struct EngineStream {
     TileParams p;
     int cdt;     // EXW_F32 / EXW_F16
-    int tma;     // stage this stream's tiles with TMA windows (else every tile reads global memory)
+    int stage;   // how this stream's windows are staged: kStageNone (every tile reads global memory), kStageTma,
+                 // kStageLoad (the loader warps)
     int nregions, ntiles, nfix;
 };
+constexpr int kStageNone = 0, kStageTma = 1, kStageLoad = 2;
 struct EngineSeg {
     int start;         // first queue index of the segment
     uint16_t stream;
@@ -67,6 +75,7 @@ struct EngineSeg {
 };
 struct EngineParams {
     int n, nseg, total, inject;
+    int loaders;      // some stream is staged by the loader warps (LOAD kernels)
     int pair_smooth;  // two smooth tiles of a stream that follow each other share one slot
     uint64_t ahead;  // streams whose bounds and plans were computed before the launch (bit s = stream s)
     uint32_t *queue, *status;
@@ -106,6 +115,14 @@ struct alignas(16) TileSlot {
     };
 };
 
+// What the loader warps stage into a slot's buffer.
+struct LoadJob {
+    int what;  // kLoadNothing, kLoadColor (one window at the buffer's start), kLoadPair (two), kLoadAll (depth, motion,
+               // colour), kLoadEnd (the end slot)
+    int stream, x0, y0, x1, y1;  // window origins (x1, y1: the second one)
+};
+constexpr int kLoadNothing = 0, kLoadColor = 1, kLoadPair = 2, kLoadAll = 3, kLoadEnd = 4;
+
 constexpr int kWindowBytes = 64512;  // both window shapes (56 x 48 FP32, 64 x 56 FP16) hold 64,512 bytes
 static_assert(64 * 16 * kConsumerWarps <= kWindowBytes, "the coarse pass's per-warp scratch fits one buffer");
 static_assert(sizeof(SplatTile) == sizeof(float4), "the candidate list doubles as one float4 per consumer thread");
@@ -127,7 +144,8 @@ struct EngineSmem {
     uint32_t ncand;
     uint32_t snext[2];                               // the next splat chunk of the tile in each buffer
     int abort;                                       // a bounded wait ran out: every warp leaves
-    uint64_t full[2], empty[2];
+    LoadJob job[2];                                  // and the loader warps' part of it
+    uint64_t full[2], empty[2], go[2];
 };
 
 // The shared memory stays within the 196 KB carve-out (with the 1 KB the system keeps per CTA): the next larger one
@@ -223,6 +241,12 @@ __device__ __forceinline__ bool stage_wait(const uint32_t *counter, uint32_t tar
     }
 }
 
+// The loader warps' part of the slot in buffer b (one thread; the buffer is free).
+__device__ __forceinline__ void hand_job(EngineSmem &s, int b, const LoadJob &job) {
+    s.job[b] = job;
+    mbar_arrive(&s.go[b]);
+}
+
 struct QueueItem {
     int item, stream, stage, local;  // item >= total: no more items
 };
@@ -239,7 +263,7 @@ __device__ __forceinline__ QueueItem decode(const EngineParams &ep, int item, in
     return q;
 }
 
-template <int SHAPE>
+template <bool LOAD, int SHAPE>
 __device__ inline void engine_producer(EngineSmem &s, const EngineParams &ep) {
     using WS = WinShape<SHAPE>;
     constexpr int kWords = (int)(sizeof(TilePlan) / 4);
@@ -346,6 +370,7 @@ __device__ inline void engine_producer(EngineSmem &s, const EngineParams &ep) {
         if (item >= ep.total) {
             if (lane == 0) {
                 sl.kind = kSlotEnd;
+                if constexpr (LOAD) hand_job(s, b, LoadJob{kLoadEnd, 0, 0, 0, 0, 0});
                 mbar_arrive(&s.full[b]);
             }
             return;
@@ -353,13 +378,16 @@ __device__ inline void engine_producer(EngineSmem &s, const EngineParams &ep) {
         const int kind = stage == 0 ? kSlotBounds : stage == 1 ? kSlotPlans : stage == 2 ? kSlotTile : kSlotFixup;
         int mode = -1, wx0 = 0, wy0 = 0, wx02 = 0, wy02 = 0;
         bool pair = false;
+        if constexpr (LOAD) {
+            if (kind != kSlotTile && lane == 0) hand_job(s, b, LoadJob{kLoadNothing, 0, 0, 0, 0, 0});
+        }
         if (kind == kSlotTile) {
             if (!have_word) word = lane < kWords ? __ldcg(reinterpret_cast<const int *>(p.plans + local) + lane) : 0;
             mode = __shfl_sync(0xFFFFFFFFu, word, 0);
             wx0 = __shfl_sync(0xFFFFFFFFu, word, 1);
             wy0 = __shfl_sync(0xFFFFFFFFu, word, 2);
             const int ndesc = __shfl_sync(0xFFFFFFFFu, word, 3);
-            if (!st.tma && mode != 4) mode = 3;  // no window: every tile reads global memory
+            if (st.stage == kStageNone && mode != 4) mode = 3;  // no window: every tile reads global memory
             // two smooth tiles in a row (the second one's plan already read): one slot, one pass of the pipeline
             pair = ep.pair_smooth && mode == 5 && nhave && nxt.stream == stream && nxt.stage == 2 &&
                    __shfl_sync(0xFFFFFFFFu, nword, 0) == 5;
@@ -369,7 +397,15 @@ __device__ inline void engine_producer(EngineSmem &s, const EngineParams &ep) {
             }
             // the window copies first: they land while the rest of the slot is written (the slot's arrival, last,
             // completes the phase together with their bytes)
-            if (lane == 0 && (mode == 0 || mode == 1 || mode == 5)) {
+            const bool windowed = mode == 0 || mode == 1 || mode == 5;
+            if constexpr (LOAD) {
+                const int what = !windowed || st.stage != kStageLoad ? kLoadNothing
+                                 : mode != 5                         ? kLoadAll
+                                 : pair                              ? kLoadPair
+                                                                     : kLoadColor;
+                if (lane == 0) hand_job(s, b, LoadJob{what, stream, wx0, wy0, wx02, wy02});
+            }
+            if (lane == 0 && windowed && (!LOAD || st.stage == kStageTma)) {
                 const CUtensorMap *m = ep.maps[stream];
                 unsigned char *wb = s.win[b];
                 // a window holds npx pixels: depth (4 B), motion (8 B), colour (3 c B) planes in this order
@@ -449,6 +485,87 @@ __device__ inline void engine_producer(EngineSmem &s, const EngineParams &ep) {
             desc0 = ndesc0;
             desc1 = ndesc1;
         }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// Loaders
+// ------------------------------------------------------------------------------------------------------------
+template <int N>
+__device__ __forceinline__ void copy_async(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
+}
+
+// Rows w, w + kLoaderWarps, ... of one plane of a window into dst (WY rows of WX elements), by loader warp w, in copies
+// of N bytes (WX elements are at most two per lane).  Pixels outside the frame are left as they are: no tile uses them.
+template <int N, typename CT, int WX, int WY>
+__device__ __forceinline__ void load_rows(CT *dst, const CT *plane, int W, int H, int x0, int y0, int w, int lane) {
+    constexpr int kPer = N / (int)sizeof(CT);   // elements per copy
+    static_assert(WX % kPer == 0 && WX / kPer <= 64, "two copies per lane and row at most");
+    const int q0 = kPer * lane, q1 = kPer * (lane + 32);
+    const bool in0 = q0 < WX && (unsigned)(x0 + q0) < (unsigned)W;
+    const bool in1 = q1 < WX && (unsigned)(x0 + q1) < (unsigned)W;
+    int r = w;
+    while (y0 + r < 0) r += kLoaderWarps;
+    const int rows = min(WY, H - y0);
+    const CT *src = plane + ((ptrdiff_t)(y0 + r) * W + x0 + q0);
+    uint32_t d = smem_addr(dst + r * WX + q0);
+#pragma unroll 4
+    for (; r < rows; r += kLoaderWarps) {
+        if (in0) copy_async<N>(d, src);
+        if (WX > 32 * kPer && in1) copy_async<N>(d + 32 * N, src + 32 * kPer);
+        src += (ptrdiff_t)kLoaderWarps * W;
+        d += kLoaderWarps * WX * (uint32_t)sizeof(CT);
+    }
+}
+
+// A plane's rows in the widest copies its address and row length allow (x0 is a multiple of 16 bytes).
+template <typename CT, int WX, int WY>
+__device__ __forceinline__ void load_plane(CT *dst, const CT *plane, int W, int H, int x0, int y0, int w, int lane) {
+    const uint32_t odd = ((uint32_t)(uintptr_t)plane | (uint32_t)W * (uint32_t)sizeof(CT)) & 7u;
+    if (odd == 0u) load_rows<8, CT, WX, WY>(dst, plane, W, H, x0, y0, w, lane);
+    else load_rows<4, CT, WX, WY>(dst, plane, W, H, x0, y0, w, lane);
+}
+
+template <typename CT, int WX, int WY>
+__device__ __forceinline__ void load_window(unsigned char *buf, const TileParams &p, const LoadJob &job, int w, int lane) {
+    constexpr int kN = WX * WY;
+    const size_t plane = (size_t)p.W * p.H;
+    CT *col = reinterpret_cast<CT *>(buf);
+    if (job.what == kLoadAll) {
+        float *f = reinterpret_cast<float *>(buf);
+        load_plane<float, WX, WY>(f, p.depth, p.W, p.H, job.x0, job.y0, w, lane);
+        load_plane<float, WX, WY>(f + kN, p.mv, p.W, p.H, job.x0, job.y0, w, lane);
+        load_plane<float, WX, WY>(f + 2 * kN, p.mv + plane, p.W, p.H, job.x0, job.y0, w, lane);
+        col = reinterpret_cast<CT *>(f + 3 * kN);
+    }
+#pragma unroll 1
+    for (int t = 0; t < (job.what == kLoadPair ? 2 : 1); ++t) {
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c)
+            load_plane<CT, WX, WY>(col + (3 * t + c) * kN, (const CT *)p.color + c * plane, p.W, p.H,
+                                   t ? job.x1 : job.x0, t ? job.y1 : job.y0, w, lane);
+    }
+}
+
+// Every loader thread takes every slot: it copies its rows, waits for them and arrives at the slot's full barrier, which
+// counts the producer and every loader thread.
+template <int SHAPE>
+__device__ inline void engine_loader(EngineSmem &s, const EngineParams &ep) {
+    using WS = WinShape<SHAPE>;
+    const int w = (int)(threadIdx.x - kConsumerThreads - 32) >> 5, lane = threadIdx.x & 31;
+    for (uint32_t i = 0;; ++i) {
+        const int b = (int)(i & 1u);
+        if (!mbar_wait_or_abort(&s.go[b], (i >> 1) & 1u, &s.abort, kConsumerWaitNs)) return;
+        const LoadJob job = s.job[b];
+        if (job.what != kLoadNothing && job.what != kLoadEnd) {
+            const EngineStream &st = ep.st[job.stream];
+            if (st.cdt == EXW_F16) load_window<__half, WS::xf16, WS::yf16>(s.win[b], st.p, job, w, lane);
+            else load_window<float, WS::xf32, WS::yf32>(s.win[b], st.p, job, w, lane);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        }
+        mbar_arrive(&s.full[b]);
+        if (job.what == kLoadEnd) return;
     }
 }
 
