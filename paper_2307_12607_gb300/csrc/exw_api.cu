@@ -249,7 +249,7 @@ exw_status exw_warp(const void *color, exw_dtype cdt, const float *depth, const 
     p.out_mask[0] = mask;
     p.n5x = ceil_div(W, 32);
     p.n5y = ceil_div(H, 32);
-    return from_cuda(launch_warp_tiles(p, cdt, (cudaStream_t)stream));
+    return from_cuda(launch_warp(p, cdt, false, nullptr, nullptr, (cudaStream_t)stream));
 }
 
 exw_status exw_fill_holes(void *color, exw_dtype cdt, const uint8_t *mask, int W, int H, void *ws, size_t ws_bytes,
@@ -451,39 +451,26 @@ exw_status exw_warp_recursive(const void *color, exw_dtype cdt, const float *dep
     const void *c = color;
     const float *d = depth, *m = mv;
     cudaError_t e = cudaSuccess;
+    const bool fill = (flags & EXW_FLAG_NO_FILL) == 0;
     for (int i = 0; i < steps && e == cudaSuccess; ++i) {
-        // step i: warp the previous frame (the source for i = 0) by a quarter step of the motion it carries
-        e = launch_clear_keys(keys, (size_t)W * H, s);
-        if (e == cudaSuccess) e = launch_splat_global(d, m, W, H, 1, 2, keys, s);
-        TileParams p{};
+        // step i: warp the previous frame (the source for i = 0) by a quarter step of the motion it carries; one
+        // kernel gathers, fills and carries (the depth and motion of the next step)
+        TileParams p = tile_params(fl, fws, W, H, 1, 2, 1, 0);
         p.color = c;
         p.depth = d;
         p.mv = m;
         p.keys = keys;
-        p.W = W;
-        p.H = H;
-        p.nfrac = 1;
-        p.L = 2;
-        p.k0 = 1;
         p.out_color[0] = out[i].color;
         p.out_mask[0] = out[i].mask;
-        p.n5x = ceil_div(W, kFillTileSide);
-        p.n5y = ceil_div(H, kFillTileSide);
-        if (e == cudaSuccess) e = launch_warp_tiles(p, cdt, s);
-        if (e == cudaSuccess && (flags & EXW_FLAG_NO_FILL) == 0) {
-            TileParams f = tile_params(fl, fws, W, H, 1, 0, 0, 0);
-            f.mask_in = out[i].mask;
-            f.out_color[0] = out[i].color;
-            e = launch_zero(fws, fl.headers + sizeof(FrameHeader), s);
-            if (e == cudaSuccess) e = launch_fill_tiles(f, cdt, s);
-            if (e == cudaSuccess) e = launch_fixup(f, cdt, s);
-        }
-        if (e == cudaSuccess && i + 1 < steps) {  // the warped frame's depth and motion for the next step
-            float *dn = (float *)(b + r.depth[i & 1]), *mn = (float *)(b + r.mv[i & 1]);
-            e = launch_carry_motion(keys, out[i].mask, d, m, W, H, dn, mn, s);
-            d = dn;
-            m = mn;
-        }
+        const bool carry = i + 1 < steps;
+        float *dn = carry ? (float *)(b + r.depth[i & 1]) : nullptr, *mn = carry ? (float *)(b + r.mv[i & 1]) : nullptr;
+        const size_t header = fill ? fl.headers + sizeof(FrameHeader) : 0;  // the fill's counters
+        e = launch_clear_keys(keys, (size_t)W * H, s, fws, header / 4);
+        if (e == cudaSuccess) e = launch_splat_global(d, m, W, H, 1, 2, keys, s);
+        if (e == cudaSuccess) e = launch_warp(p, cdt, fill, dn, mn, s);
+        if (e == cudaSuccess && fill) e = launch_fixup(p, cdt, s);
+        d = dn;
+        m = mn;
         c = out[i].color;
     }
     return from_cuda(e);

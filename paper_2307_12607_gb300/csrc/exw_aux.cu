@@ -3,9 +3,25 @@
 
 namespace exw {
 
-__global__ void clear_keys_kernel(unsigned long long *keys, size_t n) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        keys[i] = kKeyEmpty;
+// n keys (8-byte aligned) to empty, in 16-byte stores (the first and last key alone where they do not pair up), and
+// zero_words words of a frame header to zero.
+__global__ void __launch_bounds__(256) clear_keys_kernel(unsigned long long *keys, size_t n, uint32_t *zero,
+                                                         size_t zero_words) {
+    grid_dependency_wait();
+    grid_dependents_launch();  // the splat
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
+    const size_t head = ((uintptr_t)keys & 15u) ? 1 : 0, npair = (n - head) / 2;
+    ulonglong2 *pairs = reinterpret_cast<ulonglong2 *>(keys + head);
+    const ulonglong2 empty = make_ulonglong2(kKeyEmpty, kKeyEmpty);
+    size_t i0 = t;
+    for (; i0 + 3 * nt < npair; i0 += 4 * nt) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) pairs[i0 + u * nt] = empty;
+    }
+    for (; i0 < npair; i0 += nt) pairs[i0] = empty;
+    if (t == 0 && head) keys[0] = kKeyEmpty;
+    if (t == 1 && head + 2 * npair < n) keys[n - 1] = kKeyEmpty;
+    for (size_t i = t; i < zero_words; i += nt) zero[i] = 0u;
 }
 
 __global__ void zero_kernel(uint32_t *p, size_t nwords) {
@@ -13,22 +29,35 @@ __global__ void zero_kernel(uint32_t *p, size_t nwords) {
         p[i] = 0u;
 }
 
-// Stage (a) into a global key buffer: one thread per source pixel, 64-bit atomicMin at the target.
+// Stage (a) into a global key buffer: kSplatRows source pixels of one column per thread, their loads issued together,
+// and a 64-bit atomicMin at each target (a warp's 32 targets of a row mostly share sectors).
+constexpr int kSplatRows = 4;
 __global__ void __launch_bounds__(256) splat_global_kernel(const float *__restrict__ depth,
                                                            const float *__restrict__ mv, int W, int H, int k, int L,
                                                            unsigned long long *keys) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+    grid_dependency_wait();  // the keys are cleared by the kernel before
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y0 = blockIdx.y * kSplatRows;
     if (x >= W) return;
-    const size_t plane = (size_t)W * H;
-    const size_t i = (size_t)y * W + x;
-    const uint32_t db = __float_as_uint(__ldg(depth + i));
-    const uint32_t ux = __float_as_uint(__ldg(mv + i)), uy = __float_as_uint(__ldg(mv + plane + i));
-    if (!depth_ok(db) || !finite_bits(ux) || !finite_bits(uy)) return;
-    const AxisDec dx = axis_dec(ux, L), dy = axis_dec(uy, L);
-    if (!dx.land || !dy.land) return;
-    const int gx = x + axis_off(dx, k), gy = y + axis_off(dy, k);
-    if (gx < 0 || gx >= W || gy < 0 || gy >= H) return;
-    atomicMin(keys + (size_t)gy * W + gx, (unsigned long long)pack_key_global(db, (uint32_t)i));
+    const float *mvy = mv + (size_t)W * H;
+    uint32_t db[kSplatRows], ux[kSplatRows], uy[kSplatRows];
+#pragma unroll
+    for (int r = 0; r < kSplatRows; ++r) {
+        const uint32_t i = (uint32_t)min(y0 + r, H - 1) * (uint32_t)W + (uint32_t)x;
+        db[r] = __float_as_uint(__ldg(depth + i));
+        ux[r] = __float_as_uint(__ldg(mv + i));
+        uy[r] = __float_as_uint(__ldg(mvy + i));
+    }
+#pragma unroll
+    for (int r = 0; r < kSplatRows; ++r) {
+        const int y = y0 + r;
+        if (y >= H || !depth_ok(db[r]) || !finite_bits(ux[r]) || !finite_bits(uy[r])) continue;
+        const AxisDec dx = axis_dec(ux[r], L), dy = axis_dec(uy[r], L);
+        if (!dx.land || !dy.land) continue;
+        const int gx = x + axis_off(dx, k), gy = y + axis_off(dy, k);
+        if ((unsigned)gx >= (unsigned)W || (unsigned)gy >= (unsigned)H) continue;
+        atomicMin(keys + ((uint32_t)gy * (uint32_t)W + (uint32_t)gx),
+                  (unsigned long long)pack_key_global(db[r], (uint32_t)y * (uint32_t)W + (uint32_t)x));
+    }
 }
 
 // Stage (a0): one 32 x 32 source region per CTA of 4 warps (8 rows each, 24 loads in flight per thread), up to 12
@@ -89,12 +118,15 @@ static unsigned grid_for(size_t n, unsigned per_block) {
     return (unsigned)(g ? g : 1);
 }
 
-cudaError_t launch_clear_keys(uint64_t *keys, size_t n, cudaStream_t s) {
+cudaError_t launch_clear_keys(uint64_t *keys, size_t n, cudaStream_t s, void *zero, size_t zero_words) {
+    unsigned long long *const k = (unsigned long long *)keys;
+    uint32_t *const z = (uint32_t *)zero;
     timing_begin("exw_clear_keys", s);
-    clear_keys_kernel<<<grid_for(n, 256 * 4), 256, 0, s>>>((unsigned long long *)keys, n);
+    const cudaError_t e =
+        launch_dependent(clear_keys_kernel, dim3(grid_for(n, 256 * 8)), dim3(256), 0, s, k, n, z, zero_words);
     count_launch();
     timing_end("exw_clear_keys", s);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_zero(void *p, size_t bytes, cudaStream_t s) {
@@ -139,12 +171,13 @@ cudaError_t launch_carry_motion(const uint64_t *keys, const uint8_t *mask, const
 
 cudaError_t launch_splat_global(const float *depth, const float *mv, int W, int H, int k, int L, uint64_t *keys,
                                 cudaStream_t s) {
-    const dim3 g((unsigned)((W + 255) / 256), (unsigned)H, 1);
+    const dim3 g((unsigned)ceil_div(W, 256), (unsigned)ceil_div(H, kSplatRows), 1);
+    unsigned long long *const kp = (unsigned long long *)keys;
     timing_begin("exw_splat_global", s);
-    splat_global_kernel<<<g, 256, 0, s>>>(depth, mv, W, H, k, L, (unsigned long long *)keys);
+    const cudaError_t e = launch_dependent(splat_global_kernel, g, dim3(256), 0, s, depth, mv, W, H, k, L, kp);
     count_launch();
     timing_end("exw_splat_global", s);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_bounds(const float *depth, const float *mv, int W, int H, float4 *tile_bounds, float2 *tile_depth,

@@ -19,7 +19,9 @@ constexpr int kMaxFrac = 3;
 
 // Grids launched by launch_dependent: wait until the grids before this one on the stream have completed and their
 // writes are visible (at once for a grid launched without programmatic serialisation), and let the next grid be
-// scheduled (it waits in turn before touching memory).
+// scheduled (it waits in turn before touching memory).  Only a kernel that another one of the same entry point follows
+// lets it be scheduled early, and after its own wait: what a kernel reads through the read-only path was then complete
+// before its grid began, whoever launched the kernels before.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
@@ -112,20 +114,25 @@ template <> __device__ __forceinline__ float storage_round<__half>(float v) {
 // Source accessors: global memory, or a shared-memory window [x0, x0 + WX) x [y0, y0 + WY) staged by TMA.
 // ------------------------------------------------------------------------------------------------------------
 template <typename CT>
-struct GlobalAcc {
-    const CT *col;
-    const float *depth;
-    const float *mv;
-    int W;
-    size_t plane;
-    __device__ __forceinline__ size_t at(int x, int y) const { return (size_t)y * W + x; }
-    __device__ __forceinline__ size_t stride() const { return (size_t)W; }
+struct GlobalAcc {  // 32-bit element indices (a plane has at most 2^28), so an address is one wide multiply-add
+    const CT *col[3];
+    const float *depth, *mvx, *mvy;
+    uint32_t W;
+    __device__ __forceinline__ GlobalAcc(const void *color, const float *depth_, const float *mv, int W_, int H)
+        : depth(depth_), mvx(mv), W((uint32_t)W_) {
+        const size_t plane = (size_t)W_ * H;
+        mvy = mv + plane;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) col[c] = (const CT *)color + c * plane;
+    }
+    __device__ __forceinline__ uint32_t at(int x, int y) const { return (uint32_t)y * W + (uint32_t)x; }
+    __device__ __forceinline__ uint32_t stride() const { return W; }
     __device__ __forceinline__ int safe_x() const { return 0; }  // a pixel every access may use
     __device__ __forceinline__ int safe_y() const { return 0; }
-    __device__ __forceinline__ float d(size_t i) const { return __ldg(depth + i); }
-    __device__ __forceinline__ float mx(size_t i) const { return __ldg(mv + i); }
-    __device__ __forceinline__ float my(size_t i) const { return __ldg(mv + plane + i); }
-    __device__ __forceinline__ float c(int ch, size_t i) const { return load_c<CT>(col + ch * plane + i); }
+    __device__ __forceinline__ float d(uint32_t i) const { return __ldg(depth + i); }
+    __device__ __forceinline__ float mx(uint32_t i) const { return __ldg(mvx + i); }
+    __device__ __forceinline__ float my(uint32_t i) const { return __ldg(mvy + i); }
+    __device__ __forceinline__ float c(int ch, uint32_t i) const { return load_c<CT>(col[ch] + i); }
 };
 
 template <typename CT, int WX, int WY>
@@ -182,7 +189,6 @@ __device__ __forceinline__ float weight_sum(float w00, float w10, float w01, flo
 // ------------------------------------------------------------------------------------------------------------
 // Pull-push inside one 32 x 32 fill tile.  Tiles are aligned to 32, so every ancestor up to level 5 of a tile pixel
 // is computed from that tile alone; out-of-frame pixels are invalid, which reproduces the ceil-halving level sizes.
-// Warp w of 16 owns tile rows 2w and 2w+1 (lane = column).
 // ------------------------------------------------------------------------------------------------------------
 
 // Mean of the valid children, taken in the order (0,0),(0,1),(1,0),(1,1) (row, column); .w = validity.
@@ -206,64 +212,6 @@ __device__ __forceinline__ float4 shfl4_xor(float4 v, int m) {
 __device__ __forceinline__ float4 shfl4_idx(float4 v, int src) {
     return make_float4(__shfl_sync(0xFFFFFFFFu, v.x, src), __shfl_sync(0xFFFFFFFFu, v.y, src),
                        __shfl_sync(0xFFFFFFFFu, v.z, src), __shfl_sync(0xFFFFFFFFu, v.w, src));
-}
-
-// Pyramid levels 1..5 of one 32 x 32 tile in shared memory: 16x16, 8x8, 4x4, 2x2, 1x1 nodes.
-struct TilePyr {
-    float4 l1[256];
-    float4 l2[64];
-    float4 l3[16];
-    float4 l4[4];
-    float4 l5;
-};
-
-// Build the pyramid from this thread's two pixels (tile rows 2w and 2w+1 of column lane; .w = validity) with
-// 16 warps per CTA.  Level 1 is formed in registers (warp shuffle with the neighbouring column), levels 2..5 by
-// warp 0.  Contains two block barriers, which every thread must reach.  Returns this thread's level-1 node.
-__device__ __forceinline__ float4 build_pyramid(TilePyr &t, float4 top, float4 bot) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const float4 ptop = shfl4_xor(top, 1), pbot = shfl4_xor(bot, 1);
-    const float4 n1 = (lane & 1) ? mean4(ptop, top, pbot, bot) : mean4(top, ptop, bot, pbot);
-    if ((lane & 1) == 0) t.l1[wid * 16 + (lane >> 1)] = n1;
-    __syncthreads();
-    if (wid == 0) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int node = lane + 32 * h, i = node >> 3, j = node & 7;
-            const float4 *c = t.l1 + (2 * i) * 16 + 2 * j;
-            t.l2[node] = mean4(c[0], c[1], c[16], c[17]);
-        }
-        __syncwarp();
-        if (lane < 16) {
-            const int i = lane >> 2, j = lane & 3;
-            const float4 *c = t.l2 + (2 * i) * 8 + 2 * j;
-            t.l3[lane] = mean4(c[0], c[1], c[8], c[9]);
-        }
-        __syncwarp();
-        if (lane < 4) {
-            const int i = lane >> 1, j = lane & 1;
-            const float4 *c = t.l3 + (2 * i) * 4 + 2 * j;
-            t.l4[lane] = mean4(c[0], c[1], c[4], c[5]);
-        }
-        __syncwarp();
-        if (lane == 0) t.l5 = mean4(t.l4[0], t.l4[1], t.l4[2], t.l4[3]);
-    }
-    __syncthreads();
-    return n1;
-}
-
-// Value pushed down to a pixel of this thread (tile row 2w or 2w+1, column lane): its first valid ancestor; .w = 0
-// when the whole tile is invalid.  n1 is the thread's level-1 node.
-__device__ __forceinline__ float4 push_value(const TilePyr &t, float4 n1) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (n1.w != 0.0f) return n1;
-    const float4 v2 = t.l2[(wid >> 1) * 8 + (lane >> 2)];
-    if (v2.w != 0.0f) return v2;
-    const float4 v3 = t.l3[(wid >> 2) * 4 + (lane >> 3)];
-    if (v3.w != 0.0f) return v3;
-    const float4 v4 = t.l4[(wid >> 3) * 2 + (lane >> 4)];
-    if (v4.w != 0.0f) return v4;
-    return t.l5;
 }
 
 // Ordered encoding of a non-NaN float for unsigned atomicMax: larger float <-> larger code, and 0 is below every

@@ -25,7 +25,7 @@
 // target q is the source q - o_k when that pixel is valid and carries the tile's motion, so no splat is needed.
 // Other tiles splat their candidate sources into per-fraction region keys (from the window, or from global memory
 // when the landing rectangle is wider than a window) and gather through the keys.  Every result is bit-identical
-// to the per-tile passes of exw_tile.cuh (same arithmetic in the same order).
+// to the staged kernels of exw_fwd.cu (same arithmetic in the same order).
 #pragma once
 
 #include "exw_items.cuh"
@@ -1003,21 +1003,6 @@ __device__ __forceinline__ void gather_block(const uint64_t *keys, const Acc &a,
 // Epilogue: fill (pull-push levels 1..5 of the tile, Sec. IV-B stage (c)) and stores
 // ------------------------------------------------------------------------------------------------------------
 
-// Levels 3, 4 and 5 of a group's tile from its level-2 nodes (one warp; every lane returns l5, lane L < 16 its
-// level-3 node L = (L >> 2, L & 3), lane L < 4 its level-4 node).
-__device__ __forceinline__ void upper_levels(const float4 *l2, float4 &l3, float4 &l4, float4 &l5) {
-    const int lane = threadIdx.x & 31;
-    const int L = lane & 15;
-    const int I = L >> 2, J = L & 3;
-    const float4 *c = l2 + (2 * I) * 8 + 2 * J;
-    l3 = mean4(c[0], c[1], c[8], c[9]);
-    const int b4 = 8 * ((lane & 3) >> 1) + 2 * (lane & 1);
-    const float4 q0 = shfl4_idx(l3, b4), q1 = shfl4_idx(l3, b4 + 1), q2 = shfl4_idx(l3, b4 + 4),
-                 q3 = shfl4_idx(l3, b4 + 5);
-    l4 = mean4(q0, q1, q2, q3);
-    l5 = mean4(shfl4_idx(l4, 0), shfl4_idx(l4, 1), shfl4_idx(l4, 2), shfl4_idx(l4, 3));
-}
-
 // upper_levels through shared memory, for the fill of a tile: level-2 node (i, j) at l2[32 i + j] (row i in warp
 // i's scratch), up 20 float4 of the warp's own scratch (level 3, then level 4).  Every lane returns l5, the level-3
 // node (w >> 1, bx >> 2) and the level-4 node (w >> 2, bx >> 3) above its block; the same nodes and order as
@@ -1552,7 +1537,7 @@ __device__ __forceinline__ void tile_group(EngineSmem &s, const TileSlot &sl, co
         const WinAcc<CT, WX, WY> wa{&win, wx0, wy0};
         gather_block<CT>(key[kk], wa, d, k, TX, TY, bx, by, c, m);
     } else if (mode == 2 || mode == 3) {
-        const GlobalAcc<CT> ga{(const CT *)p.color, p.depth, p.mv, d.W, (size_t)d.W * d.H};
+        const GlobalAcc<CT> ga(p.color, p.depth, p.mv, d.W, d.H);
         gather_block<CT>(key[kk], ga, d, k, TX, TY, bx, by, c, m);
     } else {  // 4: nothing lands
 #pragma unroll

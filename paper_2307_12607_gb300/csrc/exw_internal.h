@@ -173,7 +173,8 @@ inline int win_y(int shape, exw_dtype cdt) {
 }
 
 // Launchers (exw_fwd.cu, exw_aux.cu, exw_bwd.cu).  Each returns the launch error.
-cudaError_t launch_clear_keys(uint64_t *keys, size_t n, cudaStream_t s);
+// Clears n keys to empty and, where given, zero_words 32-bit words at zero (one launch for both).
+cudaError_t launch_clear_keys(uint64_t *keys, size_t n, cudaStream_t s, void *zero = nullptr, size_t zero_words = 0);
 cudaError_t launch_zero(void *p, size_t bytes, cudaStream_t s);
 cudaError_t launch_carry_motion(const uint64_t *keys, const uint8_t *mask, const float *depth, const float *mv,
                                 int W, int H, float *depth_out, float *mv_out, cudaStream_t s);
@@ -196,7 +197,10 @@ cudaError_t launch_color_mse(const void *a, const void *b, exw_dtype cdt, int W,
                              cudaStream_t s, bool psnr = false);
 cudaError_t launch_ssim(const void *a, const void *b, exw_dtype cdt, int W, int H, double *out, void *ws,
                         cudaStream_t s);
-cudaError_t launch_warp_tiles(const TileParams &p, exw_dtype cdt, cudaStream_t s);
+// Stage (b) of one fraction; with fill also stage (c) but its coarse fix-up, with depth_out also what
+// exw_carry_motion writes (depth_out, mv_out).
+cudaError_t launch_warp(const TileParams &p, exw_dtype cdt, bool fill, float *depth_out, float *mv_out,
+                        cudaStream_t s);
 cudaError_t launch_fill_tiles(const TileParams &p, exw_dtype cdt, cudaStream_t s);
 cudaError_t launch_fixup(const TileParams &p, exw_dtype cdt, cudaStream_t s);
 cudaError_t launch_l2_loss(const void *out, const void *target, exw_dtype cdt, const uint8_t *mask, int W, int H,

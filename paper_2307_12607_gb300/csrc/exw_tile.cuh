@@ -1,10 +1,6 @@
-// exw_tile.cuh -- per-tile passes shared by the forward kernels (one 32 x 32 target tile Q per CTA iteration).
-//
-// A tile's keys cover Q plus a one-pixel ring R (the crack rule reads 4-neighbours).  The splat takes every
-// source pixel that can land in R -- found from the 8 x 8 motion bounds -- either from a TMA-staged shared-memory
-// window or from global memory; the gather reads through the matching accessor.  Per fraction the tile is then
-// gathered, hole-marked, filled from pyramid levels 1..5 and stored.  A CTA has 16 warps; warp w handles tile rows
-// 2w and 2w+1 with lane = column, so each row access is one 128-byte line.
+// exw_tile.cuh -- what the per-tile kernels and the engine share: the reach of a target tile under the motion bounds,
+// and the fill's pull-push pyramid (levels 1 to 5 of a 32 x 32 tile, the coarse levels above them, the bookkeeping of
+// tiles without a valid pixel).
 #pragma once
 
 #include "exw_device.cuh"
@@ -15,23 +11,10 @@ namespace exw {
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 
-struct TileSmem {
-    uint64_t key[kMaxFrac][kRegionN];  // region keys; in uniform tiles reused as depth words (uint32 per cell)
-    TilePyr pyr;                       // pyramid levels 1..5 of the fraction being filled
-    uint32_t cand[kThreads];
-    uint32_t ncand;
-    int tile, last, flag;
-    uint64_t mbar;
-};
-
 struct Rect {
     int x0, x1, y0, y1;
     __device__ __forceinline__ bool empty() const { return x1 < x0 || y1 < y0; }
 };
-
-__device__ __forceinline__ void init_keys(TileSmem &s, int nfrac) {
-    for (int i = threadIdx.x; i < nfrac * kRegionN; i += blockDim.x) (&s.key[0][0])[i] = kKeyEmpty;
-}
 
 // The block range that can reach region R (RX0, RY0 .. +33) under the frame-wide motion bounds, for fractions
 // k0 .. k0+nfrac-1.  Returns false when nothing can land anywhere.
@@ -75,113 +58,6 @@ __device__ __forceinline__ void bounds_offsets(const BoundsDec &d, int k, int &o
     ox1 = axis_off(d.x1, k);
     oy0 = axis_off(d.y0, k);
     oy1 = axis_off(d.y1, k);
-}
-
-// Splat one source pixel (x, y) for the fractions in fm into the region keys.
-__device__ __forceinline__ void splat_pixel(TileSmem &s, const TileParams &p, int x, int y, uint32_t db, uint32_t ux,
-                                            uint32_t uy, uint32_t fm, int RX0, int RY0) {
-    if (!depth_ok(db) || !finite_bits(ux) || !finite_bits(uy)) return;
-    const AxisDec dx = axis_dec(ux, p.L), dy = axis_dec(uy, p.L);
-    if (!dx.land || !dy.land) return;
-    const uint64_t key = pack_key_local(db, x, y);
-    for (int kk = 0; kk < p.nfrac; ++kk) {
-        if (!(fm & (1u << kk))) continue;
-        const int k = p.k0 + kk;
-        const int gx = x + axis_off(dx, k), gy = y + axis_off(dy, k);
-        if ((unsigned)gx >= (unsigned)p.W || (unsigned)gy >= (unsigned)p.H) continue;
-        const int rx = gx - RX0, ry = gy - RY0;
-        if ((unsigned)rx < (unsigned)kRegion && (unsigned)ry < (unsigned)kRegion)
-            atomicMin((unsigned long long *)&s.key[kk][ry * kRegion + rx], (unsigned long long)key);
-    }
-}
-
-// Splat from a staged window: every pixel of rectangle U (inside the window) for the fractions in fm.
-template <typename CT, int WX, int WY>
-__device__ __forceinline__ void splat_window(TileSmem &s, const TileParams &p, const WinAcc<CT, WX, WY> &a, Rect U,
-                                             uint32_t fm, int RX0, int RY0) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int y = U.y0 + wid; y <= U.y1; y += kWarps) {
-        for (int x = U.x0 + lane; x <= U.x1; x += 32) {
-            const int i = a.at(x, y);
-            splat_pixel(s, p, x, y, __float_as_uint(a.w->depth[i]), __float_as_uint(a.w->mv[0][i]),
-                        __float_as_uint(a.w->mv[1][i]), fm, RX0, RY0);
-        }
-    }
-}
-
-// Splat from global memory: candidate 8 x 8 tiles (those whose bounds reach R), 64 threads per candidate.
-__device__ inline void splat_global(TileSmem &s, const TileParams &p, int RX0, int RY0) {
-    const int tid = threadIdx.x;
-    int bx0, bx1, by0, by1;
-    if (!frame_window(p, RX0, RY0, bx0, bx1, by0, by1)) return;
-    const int nbxr = bx1 - bx0 + 1;
-    const int total = nbxr * (by1 - by0 + 1);
-    const size_t plane = (size_t)p.W * p.H;
-    for (int base = 0; base < total; base += kThreads) {
-        if (tid == 0) s.ncand = 0u;
-        __syncthreads();
-        const int idx = base + tid;
-        if (idx < total) {
-            const int by = by0 + idx / nbxr, bx = bx0 + idx % nbxr;
-            const float4 b = __ldcg(p.tile_bounds + (size_t)by * p.nbx + bx);
-            if (b.x <= b.y) {
-                uint32_t fm = 0;
-                const BoundsDec bd = bounds_dec(b, p.L);
-                for (int kk = 0; kk < p.nfrac; ++kk) {
-                    int ox0, ox1, oy0, oy1;
-                    bounds_offsets(bd, p.k0 + kk, ox0, ox1, oy0, oy1);
-                    const int tx0 = 8 * bx + ox0, tx1 = 8 * bx + 7 + ox1;
-                    const int ty0 = 8 * by + oy0, ty1 = 8 * by + 7 + oy1;
-                    if (tx1 >= RX0 && tx0 < RX0 + kRegion && ty1 >= RY0 && ty0 < RY0 + kRegion) fm |= 1u << kk;
-                }
-                if (fm) {
-                    const uint32_t slot = atomicAdd(&s.ncand, 1u);
-                    s.cand[slot] = (uint32_t)bx | ((uint32_t)by << 12) | (fm << 24);
-                }
-            }
-        }
-        __syncthreads();
-        const int nc = (int)s.ncand;
-        for (int c0 = 0; c0 < nc; c0 += kThreads / 64) {
-            const int ci = c0 + (tid >> 6);
-            if (ci < nc) {
-                const uint32_t e = s.cand[ci];
-                const int bx = (int)(e & 0xFFFu), by = (int)((e >> 12) & 0xFFFu);
-                const int x = 8 * bx + (tid & 7), y = 8 * by + ((tid >> 3) & 7);
-                if (x < p.W && y < p.H) {
-                    const size_t i = (size_t)y * p.W + x;
-                    splat_pixel(s, p, x, y, __float_as_uint(__ldg(p.depth + i)), __float_as_uint(__ldg(p.mv + i)),
-                                __float_as_uint(__ldg(p.mv + plane + i)), e >> 24, RX0, RY0);
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// Uniform tile: every source pixel that can land in R moves by one motion (mx, my), so for fraction kk the target
-// q can only receive the source q - o, and does when that pixel has a valid depth and exactly that motion (a pixel
-// there with another motion sits in a tile whose bounds cannot reach R, so it lands elsewhere).  Writes its depth
-// word, or all ones for an empty target, for every cell of R: the key words the splat would produce.
-template <typename CT, int WX, int WY>
-__device__ __forceinline__ void uniform_words(uint32_t *dw, const TileParams &p, const WinAcc<CT, WX, WY> &a, int ox,
-                                             int oy, float mx, float my, int RX0, int RY0) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {  // 34 x 34 cells: rows wid + 16 (i >> 1), columns lane + 32 (i & 1)
-        const int ry = wid + kWarps * (i >> 1), rx = lane + 32 * (i & 1);
-        if (ry >= kRegion || rx >= kRegion) continue;
-        const int qx = RX0 + rx, qy = RY0 + ry;
-        const int px = qx - ox, py = qy - oy;
-        uint32_t w = 0xFFFFFFFFu;
-        if ((unsigned)qx < (unsigned)p.W && (unsigned)qy < (unsigned)p.H && (unsigned)px < (unsigned)p.W &&
-            (unsigned)py < (unsigned)p.H) {
-            const int ai = a.at(px, py);
-            const uint32_t db = __float_as_uint(a.w->depth[ai]);
-            if (depth_ok(db) && a.w->mv[0][ai] == mx && a.w->mv[1][ai] == my) w = db;
-        }
-        dw[ry * kRegion + rx] = w;
-    }
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -267,175 +143,77 @@ __device__ __forceinline__ void tile_done(const TileParams &p, int *last) {
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Fill and store one fraction of a tile: c[j] (.w = validity) are this thread's two pixels (tile rows 2w + j,
-// column lane), m[j] their mask bytes (for pixels in the frame).  write_valid: store valid pixels too (fused pass)
-// or only the filled holes (in-place fill); write_mask: store the mask.  Contains two block barriers.
+// Pull-push of one 32 x 32 tile by kTileThreads threads: lane = column, warp w the rows 2w and 2w + 1, so every row
+// access is one line and a thread's pixels need no index arithmetic of their own.  Level 1 of two columns' pixels is
+// formed with a shuffle, levels 2 to 5 by warp 0 from the tile's 256 level-1 nodes in shared memory; the others wait
+// for them only where some hole has no valid level-1 ancestor.
 // ------------------------------------------------------------------------------------------------------------
-template <typename CT>
-__device__ __forceinline__ void fill_store(const TileParams &p, TilePyr &pyr, const float4 c[2], const uint8_t m[2],
-                                           int kk, int X0, int Y0, int tile, bool write_valid, bool write_mask) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const size_t plane = (size_t)p.W * p.H;
-    const int gx = X0 + lane;
-    CT *oc = (CT *)p.out_color[kk];
-    const float4 n1 = build_pyramid(pyr, c[0], c[1]);
-    const bool tile_valid = pyr.l5.w != 0.0f;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int gy = Y0 + 2 * wid + j;
-        if (gx >= p.W || gy >= p.H) continue;
-        const size_t q = (size_t)gy * p.W + gx;
-        if (write_mask) p.out_mask[kk][q] = m[j];
-        if (!tile_valid) continue;  // every pixel is a hole; the coarse fix-up writes them
-        const bool hole = m[j] != 0;
-        if (!hole && !write_valid) continue;
-        const float4 v = hole ? push_value(pyr, n1) : c[j];
-        oc[q] = to_storage<CT>(v.x);
-        oc[plane + q] = to_storage<CT>(v.y);
-        oc[2 * plane + q] = to_storage<CT>(v.z);
-    }
-    if (threadIdx.x == 0) publish_node(p, pyr.l5, kk, tile);
-}
+constexpr int kTileRows = 2;                              // rows per warp
+constexpr int kTileThreads = kFillTile / kTileRows * 32;  // 512
 
-// ------------------------------------------------------------------------------------------------------------
-// Winner sources of a region cell r: the splat keys, or (uniform tiles) depth words plus one whole-pixel offset.
-// ------------------------------------------------------------------------------------------------------------
-struct KeySource {
-    static constexpr bool kUniform = false;
-    const uint32_t *w;  // the keys as 32-bit words: 2r = (y << 14) | x, 2r + 1 = depth bits
-    float mx, my;       // unused
-    int ox, oy;         // unused
-    __device__ __forceinline__ uint32_t dword(int r) const { return w[2 * r + 1]; }
-    __device__ __forceinline__ void winner(int r, int, int, int &px, int &py) const {
-        const uint32_t lo = w[2 * r];
-        px = (int)(lo & 0x3FFFu);
-        py = (int)(lo >> 14);
-    }
-};
-struct UniformSource {
-    static constexpr bool kUniform = true;
-    const uint32_t *w;  // depth word per cell
-    float mx, my;       // the tile's one motion
-    int ox, oy;         // whole-pixel offset of the fraction
-    __device__ __forceinline__ uint32_t dword(int r) const { return w[r]; }
-    __device__ __forceinline__ void winner(int, int gx, int gy, int &px, int &py) const {
-        px = gx - ox;
-        py = gy - oy;
-    }
+struct TilePyramid {
+    float4 l1[256], l2[64], l3[16], l4[4], l5;
 };
 
-// ------------------------------------------------------------------------------------------------------------
-// Stage (b) + (c) of one fraction of a tile, from the winners of the region, through accessor a.  With FILL,
-// contains the two barriers of the pyramid.
-// ------------------------------------------------------------------------------------------------------------
-template <typename CT, bool FILL, class Acc, class Src>
-__device__ void finish_fraction(TileSmem &s, const Acc &a, const Src &src, const TileParams &p, int kk, int X0, int Y0,
-                                int tile) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int k = p.k0 + kk;
-    const size_t plane = (size_t)p.W * p.H;
-    const int gx = X0 + lane;
-    float4 c[2];
-    uint8_t m[2];
-    // The two pixels of this thread go through each step together, so their loads overlap.  Pixels without a
-    // winner (empty, crack, outside the frame) gather at a safe position and their result is discarded.
-    uint32_t dq[2];
-    int px[2], py[2];
-    bool ok[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int y = 2 * wid + j, gy = Y0 + y;
-        const bool in = gx < p.W && gy < p.H;
-        const int r = (y + 1) * kRegion + (lane + 1);
-        dq[j] = src.dword(r);
-        const bool empty = dq[j] == 0xFFFFFFFFu;
-        const bool crack = !empty && is_crack(dq[j], src.dword(r - 1), src.dword(r + 1), src.dword(r - kRegion),
-                                              src.dword(r + kRegion));
-        m[j] = !in ? (uint8_t)0 : empty ? (uint8_t)EXW_MASK_EMPTY : crack ? (uint8_t)EXW_MASK_CRACK : (uint8_t)0;
-        ok[j] = in && !empty && !crack;
-        src.winner(r, gx, gy, px[j], py[j]);
-        if (!ok[j]) {
-            px[j] = a.safe_x();
-            py[j] = a.safe_y();
-        }
-    }
-    // Residuals: one per fraction in a uniform tile, else from each winner's motion.
-    int usx = 0, usy = 0;
-    float urx = 0.0f, ury = 0.0f;
-    if (Src::kUniform) {
-        urx = residual(src.mx, k, p.L, src.ox, usx);
-        ury = residual(src.my, k, p.L, src.oy, usy);
-    }
-    decltype(a.at(0, 0)) i00[2], i10[2], i01[2], i11[2];
-    float wx0[2], wx1[2], wy0[2], wy1[2];
-    bool ex[2], ey[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        i00[j] = a.at(px[j], py[j]);
-        int sx = usx, sy = usy;
-        float rx = urx, ry = ury;
-        if (!Src::kUniform) {
-            rx = residual(a.mx(i00[j]), k, p.L, gx - px[j], sx);
-            ry = residual(a.my(i00[j]), k, p.L, Y0 + 2 * wid + j - py[j], sy);
-        }
-        wx1[j] = fabsf(rx);
-        wy1[j] = fabsf(ry);
-        wx0[j] = 1.0f - wx1[j];
-        wy0[j] = 1.0f - wy1[j];
-        ex[j] = sx != 0 && (unsigned)(px[j] + sx) < (unsigned)p.W;
-        ey[j] = sy != 0 && (unsigned)(py[j] + sy) < (unsigned)p.H;
-        i10[j] = ex[j] ? i00[j] + sx : i00[j];
-        const auto ir = sy > 0 ? i00[j] + a.stride() : i00[j] - a.stride();
-        i01[j] = ey[j] ? ir : i00[j];
-        i11[j] = (ex[j] && ey[j]) ? ir + sx : i00[j];
-    }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const float Dp = __uint_as_float(dq[j]);
-        const bool a10 = ex[j] && tap_agrees(a.d(i10[j]), Dp);
-        const bool a01 = ey[j] && tap_agrees(a.d(i01[j]), Dp);
-        const bool a11 = ex[j] && ey[j] && tap_agrees(a.d(i11[j]), Dp);
-        const float w00 = __fmul_rn(wx0[j], wy0[j]);
-        const float w10 = a10 ? __fmul_rn(wx1[j], wy0[j]) : 0.0f;
-        const float w01 = a01 ? __fmul_rn(wx0[j], wy1[j]) : 0.0f;
-        const float w11 = a11 ? __fmul_rn(wx1[j], wy1[j]) : 0.0f;
-        const float den = weight_sum(w00, w10, w01, w11);
-        float v[3];
-#pragma unroll
-        for (int ch = 0; ch < 3; ++ch) {
-            float n = __fmul_rn(w00, a.c(ch, i00[j]));
-            const float c10 = a.c(ch, i10[j]), c01 = a.c(ch, i01[j]), c11 = a.c(ch, i11[j]);
-            n = a10 ? fmaf(w10, c10, n) : n;
-            n = a01 ? fmaf(w01, c01, n) : n;
-            n = a11 ? fmaf(w11, c11, n) : n;
-            v[ch] = n;
-        }
-        const float inv = __frcp_rn(den);
-        const bool okj = ok[j];
-        c[j] = make_float4(okj ? storage_round<CT>(__fmul_rn(v[0], inv)) : 0.0f,
-                           okj ? storage_round<CT>(__fmul_rn(v[1], inv)) : 0.0f,
-                           okj ? storage_round<CT>(__fmul_rn(v[2], inv)) : 0.0f, okj ? 1.0f : 0.0f);
-    }
-    if (!FILL) {
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int gy = Y0 + 2 * wid + j;
-            if (gx >= p.W || gy >= p.H) continue;
-            const size_t q = (size_t)gy * p.W + gx;
-            CT *oc = (CT *)p.out_color[kk];
-            oc[q] = to_storage<CT>(c[j].x);
-            oc[plane + q] = to_storage<CT>(c[j].y);
-            oc[2 * plane + q] = to_storage<CT>(c[j].z);
-            p.out_mask[kk][q] = m[j];
-        }
-    } else {
-        fill_store<CT>(p, s.pyr, c, m, kk, X0, Y0, tile, true, true);
-    }
+// Levels 3, 4 and 5 of a tile from its level-2 nodes (one warp; every lane returns l5, lane L < 16 its level-3 node
+// L = (L >> 2, L & 3), lane L < 4 its level-4 node).
+__device__ __forceinline__ void upper_levels(const float4 *l2, float4 &l3, float4 &l4, float4 &l5) {
+    const int lane = threadIdx.x & 31;
+    const int L = lane & 15;
+    const int I = L >> 2, J = L & 3;
+    const float4 *c = l2 + (2 * I) * 8 + 2 * J;
+    l3 = mean4(c[0], c[1], c[8], c[9]);
+    const int b4 = 8 * ((lane & 3) >> 1) + 2 * (lane & 1);
+    const float4 q0 = shfl4_idx(l3, b4), q1 = shfl4_idx(l3, b4 + 1), q2 = shfl4_idx(l3, b4 + 4),
+                 q3 = shfl4_idx(l3, b4 + 5);
+    l4 = mean4(q0, q1, q2, q3);
+    l5 = mean4(shfl4_idx(l4, 0), shfl4_idx(l4, 1), shfl4_idx(l4, 2), shfl4_idx(l4, 3));
 }
 
-// The splat keys of fraction kk as a winner source.
-__device__ __forceinline__ KeySource key_source(const TileSmem &s, int kk) {
-    return KeySource{reinterpret_cast<const uint32_t *>(s.key[kk]), 0.0f, 0.0f, 0, 0};
+// Publishes the tile's level-5 node and replaces each hole of this thread's column (m[r] != 0) by its first valid
+// ancestor inside the tile; returns a bit per row whose pixel has a value now (the others' tile has no valid pixel:
+// the coarse fix-up writes them).  c[r].w = validity.  One block barrier, two where a hole lies that deep.
+__device__ __forceinline__ unsigned int fill_columns(const TileParams &p, TilePyramid &t, float4 (&c)[kTileRows],
+                                                     const uint8_t (&m)[kTileRows], int kk, int tile) {
+    static_assert(kTileRows == 2, "one level-1 node per column pair");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float4 o0 = shfl4_xor(c[0], 1), o1 = shfl4_xor(c[1], 1);
+    // children in the order (0,0), (0,1), (1,0), (1,1)
+    const float4 n1 = (lane & 1) ? mean4(o0, c[0], o1, c[1]) : mean4(c[0], o0, c[1], o1);
+    if ((lane & 1) == 0) t.l1[w * 16 + (lane >> 1)] = n1;
+    const bool deep = __syncthreads_or((m[0] | m[1]) != 0 && n1.w == 0.0f) != 0;
+    if (w == 0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int node = lane + 32 * h, i = node >> 3, j = node & 7;
+            const float4 *q = t.l1 + (2 * i) * 16 + 2 * j;
+            t.l2[node] = mean4(q[0], q[1], q[16], q[17]);
+        }
+        __syncwarp();
+        float4 l3, l4, l5;
+        upper_levels(t.l2, l3, l4, l5);
+        if (lane < 16) t.l3[lane] = l3;
+        if (lane < 4) t.l4[lane] = l4;
+        if (lane == 0) {
+            t.l5 = l5;
+            publish_node(p, l5, kk, tile);
+        }
+    }
+    float4 v = n1;
+    if (deep) {
+        __syncthreads();  // levels 2 to 5
+        if (v.w == 0.0f) v = t.l2[(w >> 1) * 8 + (lane >> 2)];
+        if (v.w == 0.0f) v = t.l3[(w >> 2) * 4 + (lane >> 3)];
+        if (v.w == 0.0f) v = t.l4[(w >> 3) * 2 + (lane >> 4)];
+        if (v.w == 0.0f) v = t.l5;
+    }
+    unsigned int have = 0u;
+#pragma unroll
+    for (int r = 0; r < kTileRows; ++r) {
+        if (m[r] != 0) c[r] = v;
+        have |= c[r].w != 0.0f ? 1u << r : 0u;
+    }
+    return have;
 }
 
 }  // namespace exw
