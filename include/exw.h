@@ -258,6 +258,13 @@ EXW_API exw_status exw_warp_backward(const float *grad_out, const void *color, e
                              const float *mv, const uint64_t *keys, int W, int H, int k, int denom,
                              float *grad_color, float *grad_mv, void *ws, size_t ws_bytes, exw_stream_t stream);
 
+/* exw_warp_backward with the gradients stored instead of accumulated (grad_color and grad_mv need no initialisation):
+ * the same bits as accumulating into zeros, without writing the zeros and reading them back (Sec. II-B, Sec. III-B; a
+ * library facility). */
+EXW_API exw_status exw_warp_backward_store(const float *grad_out, const void *color, exw_dtype cdt, const float *depth,
+                                   const float *mv, const uint64_t *keys, int W, int H, int k, int denom,
+                                   float *grad_color, float *grad_mv, void *ws, size_t ws_bytes, exw_stream_t stream);
+
 /* One frame of the training pass exw_warp_l2_grad (device pointers). */
 typedef struct exw_train_frame {
     exw_frame src;                     /* F_t: colour (cdt), depth, motion */
@@ -280,6 +287,11 @@ typedef struct exw_train_frame {
  * W, H, cdt, 1, nfrac) (the key planes of one frame; frames run one after another on the stream). */
 EXW_API exw_status exw_warp_l2_grad(const exw_train_frame *frames, int nframes, int nfrac, double *loss, void *ws,
                                     size_t ws_bytes, exw_stream_t stream);
+
+/* exw_warp_l2_grad with every frame's gradients stored instead of accumulated (no two frames may share a gradient
+ * buffer): the same bits as accumulating into zeros (Sec. IV-B; a library facility). */
+EXW_API exw_status exw_warp_l2_grad_store(const exw_train_frame *frames, int nframes, int nfrac, double *loss, void *ws,
+                                  size_t ws_bytes, exw_stream_t stream);
 
 /* L2 loss of a warped frame against a target over its non-hole pixels (the loss the differentiation workload
  * trains against): loss += sum over mask == 0 and 3 channels of (out - target)^2 (float32 device scalar,

@@ -39,6 +39,8 @@ PROTOTYPES = {
     "exw_warp_recursive": (I, [P, I, P, P, I, I, I, U, P, P, SZ, P]),
     "exw_ssim": (I, [P, P, I, I, I, P, P, SZ, P]),
     "exw_warp_backward": (I, [P, P, I, P, P, P, I, I, I, I, P, P, P, SZ, P]),
+    "exw_warp_backward_store": (I, [P, P, I, P, P, P, I, I, I, I, P, P, P, SZ, P]),
+    "exw_warp_l2_grad_store": (I, [P, I, I, P, P, SZ, P]),
     "exw_l2_loss_grad": (I, [P, P, I, P, I, I, P, P, P]),
     "exw_warp_l2_grad": (I, [P, I, I, P, P, SZ, P]),
     "exw_device_status": (I, [P, P]),

@@ -423,13 +423,18 @@ def exw_extrapolate_batched(streams, nfrac: int = 3, fill: bool = True, outs=Non
 
 def exw_warp_backward(grad_out, color, depth, mv, keys, k: int, denom: int = 4, grad_color=None, grad_mv=None,
                       ws=None, stream=None):
-    """Adjoint of stage (b); accumulates into (and returns) grad_color [3][H][W] and grad_mv [2][H][W] float32.
-    ``keys=None`` recomputes the keys into the workspace."""
+    """Adjoint of stage (b); accumulates into (and returns) grad_color [3][H][W] and grad_mv [2][H][W] float32
+    (new ones when both are None).  ``keys=None`` recomputes the keys into the workspace."""
     W, H = _hw(depth)
     dev = color.device
-    if grad_color is None:
+    call = lib().exw_warp_backward
+    if grad_color is None and grad_mv is None:  # stored, not accumulated into zeros
+        call = lib().exw_warp_backward_store
+        grad_color = torch.empty((3, H, W), dtype=torch.float32, device=dev)
+        grad_mv = torch.empty((2, H, W), dtype=torch.float32, device=dev)
+    elif grad_color is None:
         grad_color = torch.zeros((3, H, W), dtype=torch.float32, device=dev)
-    if grad_mv is None:
+    elif grad_mv is None:
         grad_mv = torch.zeros((2, H, W), dtype=torch.float32, device=dev)
     kptr = 0 if keys is None else _dev(keys, "keys", torch.int64, (H, W))
     wsp, wsn = 0, 0
@@ -437,13 +442,10 @@ def exw_warp_backward(grad_out, color, depth, mv, keys, k: int, denom: int = 4, 
         if ws is None:
             ws = workspace(exw_workspace_bytes(OP_WARP_BACKWARD, W, H, _cdt(color)), dev)
         wsp, wsn = ws.data_ptr(), ws.numel()
-    _check(lib().exw_warp_backward(_dev(grad_out, "grad_out", torch.float32, (3, H, W)),
-                                   _dev(color, "color", None, (3, H, W)), _cdt(color),
-                                   _dev(depth, "depth", torch.float32), _dev(mv, "mv", torch.float32, (2, H, W)),
-                                   kptr, W, H, int(k), int(denom),
-                                   _dev(grad_color, "grad_color", torch.float32, (3, H, W)),
-                                   _dev(grad_mv, "grad_mv", torch.float32, (2, H, W)), wsp, wsn,
-                                   _stream(stream, dev)))
+    _check(call(_dev(grad_out, "grad_out", torch.float32, (3, H, W)), _dev(color, "color", None, (3, H, W)),
+                _cdt(color), _dev(depth, "depth", torch.float32), _dev(mv, "mv", torch.float32, (2, H, W)), kptr, W, H,
+                int(k), int(denom), _dev(grad_color, "grad_color", torch.float32, (3, H, W)),
+                _dev(grad_mv, "grad_mv", torch.float32, (2, H, W)), wsp, wsn, _stream(stream, dev)))
     return grad_color, grad_mv
 
 
@@ -457,9 +459,14 @@ def exw_warp_l2_grad(color, depth, mv, targets, nfrac: int = 3, grad_color=None,
     F, _, H, W = (int(v) for v in color.shape)
     dev = color.device
     cdt = _cdt(color)
-    if grad_color is None:
+    call = lib().exw_warp_l2_grad
+    if grad_color is None and grad_mv is None:  # stored, not accumulated into zeros
+        call = lib().exw_warp_l2_grad_store
+        grad_color = torch.empty((F, 3, H, W), dtype=torch.float32, device=dev)
+        grad_mv = torch.empty((F, 2, H, W), dtype=torch.float32, device=dev)
+    elif grad_color is None:
         grad_color = torch.zeros((F, 3, H, W), dtype=torch.float32, device=dev)
-    if grad_mv is None:
+    elif grad_mv is None:
         grad_mv = torch.zeros((F, 2, H, W), dtype=torch.float32, device=dev)
     if loss is None:
         loss = torch.empty(F, dtype=torch.float64, device=dev)
@@ -479,8 +486,8 @@ def exw_warp_l2_grad(color, depth, mv, targets, nfrac: int = 3, grad_color=None,
             frames[f].target[j] = targets[f, j].data_ptr()
         frames[f].grad_color = grad_color[f].data_ptr()
         frames[f].grad_mv = grad_mv[f].data_ptr()
-    _check(lib().exw_warp_l2_grad(ctypes.cast(frames, ctypes.c_void_p), F, int(nfrac), loss.data_ptr(),
-                                  ws.data_ptr(), ws.numel(), _stream(stream, dev)))
+    _check(call(ctypes.cast(frames, ctypes.c_void_p), F, int(nfrac), loss.data_ptr(), ws.data_ptr(), ws.numel(),
+                _stream(stream, dev)))
     return loss, grad_color, grad_mv
 
 

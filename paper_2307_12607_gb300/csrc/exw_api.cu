@@ -476,9 +476,10 @@ exw_status exw_warp_recursive(const void *color, exw_dtype cdt, const float *dep
     return from_cuda(e);
 }
 
-exw_status exw_warp_backward(const float *grad_out, const void *color, exw_dtype cdt, const float *depth,
-                             const float *mv, const uint64_t *keys, int W, int H, int k, int denom, float *grad_color,
-                             float *grad_mv, void *ws, size_t ws_bytes, exw_stream_t stream) {
+static exw_status warp_backward(const float *grad_out, const void *color, exw_dtype cdt, const float *depth,
+                                const float *mv, const uint64_t *keys, int W, int H, int k, int denom,
+                                float *grad_color, float *grad_mv, bool store, void *ws, size_t ws_bytes,
+                                exw_stream_t stream) {
     const int L = log2_pow2(denom);
     if (!size_ok(W, H) || L < 0 || k < 0 || k > denom || !dtype_ok(cdt) || !aligned(grad_out, 4) ||
         !aligned(color, csize(cdt)) || !aligned(depth, 4) || !aligned(mv, 4) || !aligned(grad_color, 4) ||
@@ -498,11 +499,26 @@ exw_status exw_warp_backward(const float *grad_out, const void *color, exw_dtype
     } else if (entry_check() != EXW_OK) {
         return EXW_ERR_CUDA;
     }
-    return from_cuda(launch_backward(grad_out, color, cdt, depth, mv, kp, W, H, k, L, grad_color, grad_mv, s));
+    return from_cuda(launch_backward(grad_out, color, cdt, depth, mv, kp, W, H, k, L, grad_color, grad_mv, store,
+                                     s));
 }
 
-exw_status exw_warp_l2_grad(const exw_train_frame *frames, int nframes, int nfrac, double *loss, void *ws,
-                            size_t ws_bytes, exw_stream_t stream) {
+exw_status exw_warp_backward(const float *grad_out, const void *color, exw_dtype cdt, const float *depth,
+                             const float *mv, const uint64_t *keys, int W, int H, int k, int denom, float *grad_color,
+                             float *grad_mv, void *ws, size_t ws_bytes, exw_stream_t stream) {
+    return warp_backward(grad_out, color, cdt, depth, mv, keys, W, H, k, denom, grad_color, grad_mv, false, ws,
+                         ws_bytes, stream);
+}
+
+exw_status exw_warp_backward_store(const float *grad_out, const void *color, exw_dtype cdt, const float *depth,
+                                   const float *mv, const uint64_t *keys, int W, int H, int k, int denom,
+                                   float *grad_color, float *grad_mv, void *ws, size_t ws_bytes, exw_stream_t stream) {
+    return warp_backward(grad_out, color, cdt, depth, mv, keys, W, H, k, denom, grad_color, grad_mv, true, ws,
+                         ws_bytes, stream);
+}
+
+static exw_status warp_l2_grad(const exw_train_frame *frames, int nframes, int nfrac, double *loss, bool store,
+                               void *ws, size_t ws_bytes, exw_stream_t stream) {
     if (frames == nullptr || nframes < 1 || nfrac < 1 || nfrac > EXW_MAX_FRAC || !aligned(loss, 8))
         return EXW_ERR_INVALID_ARG;
     const int W = frames[0].src.W, H = frames[0].src.H;
@@ -520,8 +536,18 @@ exw_status exw_warp_l2_grad(const exw_train_frame *frames, int nframes, int nfra
     if (entry_check() != EXW_OK) return EXW_ERR_CUDA;
     cudaError_t e = cudaSuccess;
     for (int f = 0; f < nframes && e == cudaSuccess; ++f)
-        e = launch_train_frame(frames[f], nfrac, loss + f, ws, (cudaStream_t)stream);
+        e = launch_train_frame(frames[f], nfrac, loss + f, store, ws, (cudaStream_t)stream);
     return from_cuda(e);
+}
+
+exw_status exw_warp_l2_grad(const exw_train_frame *frames, int nframes, int nfrac, double *loss, void *ws,
+                            size_t ws_bytes, exw_stream_t stream) {
+    return warp_l2_grad(frames, nframes, nfrac, loss, false, ws, ws_bytes, stream);
+}
+
+exw_status exw_warp_l2_grad_store(const exw_train_frame *frames, int nframes, int nfrac, double *loss, void *ws,
+                                  size_t ws_bytes, exw_stream_t stream) {
+    return warp_l2_grad(frames, nframes, nfrac, loss, true, ws, ws_bytes, stream);
 }
 
 exw_status exw_l2_loss_grad(const void *out, const void *target, exw_dtype cdt, const uint8_t *mask, int W, int H,

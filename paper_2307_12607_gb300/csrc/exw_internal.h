@@ -188,7 +188,9 @@ cudaError_t launch_plan(const TileParams &p, exw_dtype cdt, int shape, cudaStrea
 
 size_t recursive_workspace_bytes(int W, int H);
 size_t train_workspace_bytes(int W, int H, int nfrac);
-cudaError_t launch_train_frame(const exw_train_frame &f, int nfrac, double *loss, void *ws, cudaStream_t s);
+// store: the gradients are written instead of accumulated (here and in launch_backward).
+cudaError_t launch_train_frame(const exw_train_frame &f, int nfrac, double *loss, bool store, void *ws,
+                               cudaStream_t s);
 
 // Frame statistics (exw_stats.cu): FP64 reductions into a small fixed workspace.
 size_t stats_workspace_bytes();
@@ -207,7 +209,7 @@ cudaError_t launch_l2_loss(const void *out, const void *target, exw_dtype cdt, c
                            float *grad_out, float *loss, cudaStream_t s);
 cudaError_t launch_backward(const float *grad_out, const void *color, exw_dtype cdt, const float *depth,
                             const float *mv, const uint64_t *keys, int W, int H, int k, int L, float *grad_color,
-                            float *grad_mv, cudaStream_t s);
+                            float *grad_mv, bool store, cudaStream_t s);
 
 // The fused forward pass of exw_extrapolate and exw_extrapolate_batched (exw_batched.cu): one engine launch per
 // group of at most 48 frames.  specs[i] = (source frame, its nfrac outputs).
