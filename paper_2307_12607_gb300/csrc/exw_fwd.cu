@@ -5,11 +5,15 @@
 namespace exw {
 
 // Plans: one warp per target tile (the first stream of an engine launch is planned ahead of the launch).
+// Small CTAs: a small frame's plans (240 at 640 x 360) spread over the SMs instead of sharing 15 of them, and a large
+// frame's last wave is short (4K: one frame's plans 26.5 us in CTAs of 16 warps, 24.4 in these; 640 x 360 13.1 and 11.7,
+// events around the launch).
+constexpr int kPlanThreads = 64;
 template <typename CT, int WX, int WY>
-__global__ void __launch_bounds__(kThreads) plan_kernel(TileParams p) {
+__global__ void __launch_bounds__(kPlanThreads, 16) plan_kernel(const __grid_constant__ TileParams p) {
     grid_dependency_wait();  // the bounds kernel before
     grid_dependents_launch();
-    const int tile = blockIdx.x * kWarps + (threadIdx.x >> 5);
+    const int tile = blockIdx.x * (kPlanThreads / 32) + (threadIdx.x >> 5);
     if (tile < p.n5x * p.n5y) plan_tile<CT, WX, WY>(p, tile);
 }
 
@@ -213,7 +217,7 @@ static dim3 tile_grid(const TileParams &p) { return dim3((unsigned)p.n5x, (unsig
 
 cudaError_t launch_plan(const TileParams &p, exw_dtype cdt, int shape, cudaStream_t s) {
     const int ntiles = p.n5x * p.n5y;
-    const unsigned g = (unsigned)((ntiles + kWarps - 1) / kWarps);
+    const unsigned g = (unsigned)ceil_div(ntiles, kPlanThreads / 32);
     timing_begin("exw_plan", s);
     using S0 = WinShape<0>;
     using S1 = WinShape<1>;
@@ -221,7 +225,7 @@ cudaError_t launch_plan(const TileParams &p, exw_dtype cdt, int shape, cudaStrea
                                                           : plan_kernel<__half, S0::xf16, S0::yf16>)
                                        : (cdt == EXW_F32 ? plan_kernel<float, S1::xf32, S1::yf32>
                                                           : plan_kernel<__half, S1::xf16, S1::yf16>);
-    const cudaError_t e = launch_dependent(k, dim3(g), dim3(kThreads), 0, s, p);
+    const cudaError_t e = launch_dependent(k, dim3(g), dim3(kPlanThreads), 0, s, p);
     count_launch();
     timing_end("exw_plan", s);
     return e != cudaSuccess ? e : cudaGetLastError();

@@ -9,7 +9,6 @@
 namespace exw {
 
 constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
 
 struct Rect {
     int x0, x1, y0, y1;
