@@ -46,21 +46,21 @@ __global__ void __launch_bounds__(256) splat_global_kernel(const float *__restri
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y0 = blockIdx.y * kSplatRows;
     if (x >= W) return;
     const float *mvy = mv + (size_t)W * H;
-    uint32_t db[kSplatRows], ux[kSplatRows], uy[kSplatRows];
+    const float kf = fraction_scale(k, L), limit = motion_limit(k, L);
+    uint32_t db[kSplatRows];
+    float mx[kSplatRows], my[kSplatRows];
 #pragma unroll
     for (int r = 0; r < kSplatRows; ++r) {
         const uint32_t i = (uint32_t)min(y0 + r, H - 1) * (uint32_t)W + (uint32_t)x;
         db[r] = __float_as_uint(__ldg(depth + i));
-        ux[r] = __float_as_uint(__ldg(mv + i));
-        uy[r] = __float_as_uint(__ldg(mvy + i));
+        mx[r] = __ldg(mv + i);
+        my[r] = __ldg(mvy + i);
     }
 #pragma unroll
     for (int r = 0; r < kSplatRows; ++r) {
         const int y = y0 + r;
-        if (y >= H || !depth_ok(db[r]) || !finite_bits(ux[r]) || !finite_bits(uy[r])) continue;
-        const AxisDec dx = axis_dec(ux[r], L), dy = axis_dec(uy[r], L);
-        if (!dx.land || !dy.land) continue;
-        const int gx = x + axis_off(dx, k), gy = y + axis_off(dy, k);
+        if (y >= H || !depth_ok(db[r]) || !motion_lands(mx[r], my[r], limit)) continue;
+        const int gx = x + offset_of(mx[r], kf), gy = y + offset_of(my[r], kf);
         if ((unsigned)gx >= (unsigned)W || (unsigned)gy >= (unsigned)H) continue;
         atomicMin(keys + ((uint32_t)gy * (uint32_t)W + (uint32_t)gx),
                   (unsigned long long)pack_key_global(db[r], (uint32_t)y * (uint32_t)W + (uint32_t)x));

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) bwd_tile_kernel(const __grid_c
     float lacc = 0.0f;  // this thread's loss terms (at most 5 cells x 3 fractions x 3 channels), then FP64
     for (int kk = 0; kk < a.nfrac; ++kk) {
         const int k = a.k0 + kk, L = a.L;
-        const float scale = -(float)k * pow2_neg(L);
+        const float kf = fraction_scale(k, L), limit = motion_limit(k, L), scale = -kf;
         const unsigned long long *keys = a.keys[kk];
         const void *const *gp = a.g[kk];
         int ry = tid / kRegion, rx = tid - ry * kRegion;  // cell r = tid, tid + 256, ...: 7 rows and 18 columns on
@@ -112,13 +112,11 @@ __global__ void __launch_bounds__(kBwdThreads, 4) bwd_tile_kernel(const __grid_c
             if (px >= 0 && px < W && py >= 0 && py < H) {
                 const uint32_t i = (uint32_t)py * Wu + (uint32_t)px;
                 const uint32_t db = __float_as_uint(sm.depth[e]);
-                const uint32_t ux = __float_as_uint(__ldg(a.mv[0] + i)), uy = __float_as_uint(__ldg(a.mv[1] + i));
-                if (depth_ok(db) && finite_bits(ux) && finite_bits(uy)) {
-                    const AxisDec dx = axis_dec(ux, L), dy = axis_dec(uy, L);
-                    const bool lands = dx.land && dy.land;
-                    const int ox = axis_off(dx, k), oy = axis_off(dy, k);
+                const float mx = __ldg(a.mv[0] + i), my = __ldg(a.mv[1] + i);
+                if (depth_ok(db) && motion_lands(mx, my, limit)) {
+                    const int ox = offset_of(mx, kf), oy = offset_of(my, kf);
                     const int qx = px + ox, qy = py + oy;
-                    if (lands && (unsigned)qx < (unsigned)W && (unsigned)qy < (unsigned)H) {
+                    if ((unsigned)qx < (unsigned)W && (unsigned)qy < (unsigned)H) {
                         const uint32_t q = (uint32_t)qy * Wu + (uint32_t)qx;
                         // every global load of the cell at once: q's key, the depth words of its 4-neighbours', g's
                         // inputs
@@ -137,8 +135,8 @@ __global__ void __launch_bounds__(kBwdThreads, 4) bwd_tile_kernel(const __grid_c
                             if (!is_crack(db, k0, k1, k2, k3)) {
                                 const float Dp = __uint_as_float(db);
                                 int sx, sy;
-                                const float rhox = residual(__uint_as_float(ux), k, L, ox, sx);
-                                const float rhoy = residual(__uint_as_float(uy), k, L, oy, sy);
+                                const float rhox = residual(mx, k, L, ox, sx);
+                                const float rhoy = residual(my, k, L, oy, sy);
                                 const float wx1 = fabsf(rhox), wy1 = fabsf(rhoy);
                                 const float wx0 = 1.f - wx1, wy0 = 1.f - wy1;
                                 const int tx = px + sx, ty = py + sy;
@@ -315,26 +313,25 @@ __global__ void __launch_bounds__(256) splat_multi_kernel(const float *__restric
     if (x >= W) return;
     const size_t plane = (size_t)W * H;
     const float *mvy = mv + plane;
-    uint32_t db[kSplatMultiRows], ux[kSplatMultiRows], uy[kSplatMultiRows];
+    uint32_t db[kSplatMultiRows];
+    float mx[kSplatMultiRows], my[kSplatMultiRows];
 #pragma unroll
     for (int r = 0; r < kSplatMultiRows; ++r) {
         const uint32_t i = (uint32_t)min(y0 + r, H - 1) * (uint32_t)W + (uint32_t)x;
         db[r] = __float_as_uint(__ldg(depth + i));
-        ux[r] = __float_as_uint(__ldg(mv + i));
-        uy[r] = __float_as_uint(__ldg(mvy + i));
+        mx[r] = __ldg(mv + i);
+        my[r] = __ldg(mvy + i);
     }
 #pragma unroll
     for (int r = 0; r < kSplatMultiRows; ++r) {
         const int y = y0 + r;
-        if (y >= H || !depth_ok(db[r]) || !finite_bits(ux[r]) || !finite_bits(uy[r])) continue;
-        const AxisDec dx = axis_dec(ux[r], L), dy = axis_dec(uy[r], L);
-        if (!dx.land || !dy.land) continue;
+        if (y >= H || !depth_ok(db[r]) || !motion_lands(mx[r], my[r], kMotionLimit)) continue;
         const unsigned long long key = pack_key_global(db[r], (uint32_t)y * (uint32_t)W + (uint32_t)x);
 #pragma unroll
         for (int kk = 0; kk < kMaxFrac; ++kk) {
             if (kk >= nfrac) break;
-            const int k = k0 + kk;
-            const int gx = x + axis_off(dx, k), gy = y + axis_off(dy, k);
+            const float kf = fraction_scale(k0 + kk, L);
+            const int gx = x + offset_of(mx[r], kf), gy = y + offset_of(my[r], kf);
             if ((unsigned)gx >= (unsigned)W || (unsigned)gy >= (unsigned)H) continue;
             atomicMin(keys + kk * plane + ((uint32_t)gy * (uint32_t)W + (uint32_t)gx), key);
         }

@@ -40,45 +40,38 @@ __device__ __forceinline__ float pow2_neg(int n) {  // 2^-n for n in [-126, 126]
 // ------------------------------------------------------------------------------------------------------------
 // Exact target offset off = floor(1/2 + k * mv / 2^L).
 //
-// A finite float mv is sM * 2^(e - 150) with |sM| < 2^24, so k*mv/2^L = k*sM * 2^-n with n = 150 + L - e.  For
-// k <= 64, |k*sM| < 2^30, and rounding half up is an arithmetic shift: off = (k*sM + 2^(n-1)) >> n.  For n >= 32
-// (|d| < 1/4) the same expression with n clamped to 31 gives 0, since |k*sM| < 2^30; n <= 0 means |d| >= 2^23,
-// which cannot land in any frame.  The decomposition is shared by all fractions, so each fraction costs one
-// multiply-add and one shift, without branches.
+// kf = k / 2^L is exact in float, and so is the product inside a fused multiply-add.  Adding 2^22 * 3/2 + 1/2 rounded
+// down leaves a float in [2^22, 2^23), whose last bit is worth 1/2: floor(2 (kf mv + 1/2)) / 2 above the base, and half
+// of that, rounded down once more by the shift, is floor(kf mv + 1/2).  Three instructions per axis and fraction and
+// nothing shared between them (the significand and exponent taken apart cost some ten per axis before the first).
+// Holds while |kf mv + 1/2| < 2^21; a motion of 2^20 pixels or more lands in no frame for any k >= 1 (|off| >= 2^14).
+// Engine time with the parts taken apart and with this: 4 frames of 1080p FP16 under a turning camera 423 and 392 us, the
+// 60-frame 1080p sequence 3816 and 3708, 48 streams 5253 and 5072; 8 training frames 1371 and 1319 us.
 // ------------------------------------------------------------------------------------------------------------
-struct AxisDec {
-    int sM;     // signed significand
-    int n;      // right-shift amount, clamped to [1, 31]
-    int half;   // 2^(n-1)
-    bool land;  // false when the motion is too large to land in any frame
-};
+constexpr float kOffsetBias = 6291456.5f;           // 3/2 2^22 + 1/2
+constexpr int kOffsetBase = 0x4AC00000 >> 1;        // half the bits of 3/2 2^22
+constexpr float kMotionLimit = 1048576.0f;          // 2^20
 
-__device__ __forceinline__ AxisDec axis_dec(uint32_t u, int L) {
-    const uint32_t E = (u >> 23) & 0xFFu;
-    const int M = (int)((u & 0x7FFFFFu) | (E ? 0x800000u : 0u));
-    const int n = 150 + L - (E ? (int)E : 1);
-    AxisDec d;
-    d.sM = (u >> 31) ? -M : M;
-    d.land = n > 0;
-    d.n = min(max(n, 1), 31);
-    d.half = 1 << (d.n - 1);
-    return d;
+__device__ __forceinline__ float fraction_scale(int k, int L) { return (float)k * pow2_neg(L); }
+__device__ __forceinline__ int offset_raw(float mv, float kf) {  // the offset plus kOffsetBase
+    return __float_as_int(__fmaf_rd(kf, mv, kOffsetBias)) >> 1;
 }
-
-__device__ __forceinline__ int axis_off(const AxisDec &d, int k) { return (k * d.sM + d.half) >> d.n; }
-
-__device__ __forceinline__ int axis_off_of(uint32_t bits, int k, int L) {  // for clamped bounds (always lands)
-    return axis_off(axis_dec(bits, L), k);
+__device__ __forceinline__ int offset_of(float mv, float kf) { return offset_raw(mv, kf) - kOffsetBase; }
+// The motions that can land somewhere: below 2^20 for k >= 1; k = 0 (staged entry points) leaves a pixel where it is
+// for any motion below 2^(23 + L), the range the offset is defined on.  A NaN is in neither.
+__device__ __forceinline__ float motion_limit(int k, int L) { return k == 0 ? __int_as_float((150 + L) << 23) : kMotionLimit; }
+__device__ __forceinline__ bool motion_lands(float mx, float my, float limit) {
+    return fabsf(mx) < limit && fabsf(my) < limit;
 }
 
 // Residual rho = t - k*mv/2^L for a winner displaced by the whole-pixel offset t (|rho| <= 1/2).  One fused
 // multiply-add computes the exact value rounded once, i.e. the correctly rounded residual.  Its sign is exact
-// except when |rho| < 2^-150 rounds to zero, which needs t = 0 and a subnormal mv; then rho = -d has the sign of
+// except when |rho| < 2^-150 rounds to zero, which needs t = 0 and a subnormal mv; with t = 0 the sign is that of
 // -mv.  sgn is -1, 0 or +1.
 __device__ __forceinline__ float residual(float mv, int k, int L, int t, int &sgn) {
     const float r = fmaf(-(float)k * pow2_neg(L), mv, (float)t);
-    sgn = (r > 0.0f) - (r < 0.0f);
-    if (sgn == 0 && t == 0 && k != 0 && mv != 0.0f) sgn = mv > 0.0f ? -1 : 1;
+    const float s = t == 0 && k != 0 ? -mv : r;
+    sgn = (s > 0.0f) - (s < 0.0f);
     return r;
 }
 

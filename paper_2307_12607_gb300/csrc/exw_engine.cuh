@@ -203,7 +203,8 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t *mbar, uint32_t pari
 __device__ __forceinline__ void uniform_frac(UniformFrac &u, const TileParams &p, uint32_t umx, uint32_t umy, int kk,
                                              int j) {
     const int k = p.k0 + kk;
-    const int ox = axis_off_of(umx, k, p.L), oy = axis_off_of(umy, k, p.L);
+    const float kf = fraction_scale(k, p.L);
+    const int ox = offset_of(__uint_as_float(umx), kf), oy = offset_of(__uint_as_float(umy), kf);
     int sx, sy;
     const float rx = residual(__uint_as_float(umx), k, p.L, ox, sx);
     const float ry = residual(__uint_as_float(umy), k, p.L, oy, sy);
@@ -713,21 +714,47 @@ __device__ __forceinline__ void uniform_block_any(const Window<CT, WX, WY> &w, i
 // ------------------------------------------------------------------------------------------------------------
 // Tiles through splat keys (modes 1-3)
 // ------------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void engine_splat_pixel(uint64_t (*key)[kRegionN], const FrameDims &p, int x, int y,
-                                                   uint32_t db, uint32_t ux, uint32_t uy, uint32_t fm, int RX0,
-                                                   int RY0) {
-    if (!depth_ok(db) || !finite_bits(ux) || !finite_bits(uy)) return;
-    const AxisDec dx = axis_dec(ux, p.L), dy = axis_dec(uy, p.L);
-    if (!dx.land || !dy.land) return;
+
+// The cells of the region R (from (RX0, RY0)) that lie in the frame: columns x0 .. x0 + nx - 1, rows likewise.
+struct RegionClip {
+    int RX0, RY0, x0, y0, nx, ny;
+    __device__ __forceinline__ RegionClip(const FrameDims &d, int RX0_, int RY0_) : RX0(RX0_), RY0(RY0_) {
+        x0 = max(0, -RX0);
+        y0 = max(0, -RY0);
+        nx = min(kRegion, d.W - RX0) - x0;
+        ny = min(kRegion, d.H - RY0) - y0;
+    }
+    // The key of cell (rx, ry) takes kv where the cell is one of them.
+    __device__ __forceinline__ void put(uint64_t *key, int rx, int ry, uint64_t kv) const {
+        if ((unsigned)(rx - x0) < (unsigned)nx && (unsigned)(ry - y0) < (unsigned)ny)
+            atomicMin((unsigned long long *)&key[ry * kRegion + rx], (unsigned long long)kv);
+    }
+};
+
+// One source pixel into the keys of the fractions in fm.
+__device__ __forceinline__ void engine_splat_pixel(uint64_t (*key)[kRegionN], const FrameDims &p,
+                                                   const RegionClip &clip, int x, int y, uint32_t db, float mx,
+                                                   float my, uint32_t fm) {
+    if (!depth_ok(db) || !motion_lands(mx, my, kMotionLimit)) return;
     const uint64_t kv = pack_key_local(db, x, y);
-    for (int kk = 0; kk < p.nfrac; ++kk) {
+    const int cx = x - clip.RX0 - kOffsetBase, cy = y - clip.RY0 - kOffsetBase;
+#pragma unroll
+    for (int kk = 0; kk < kMaxFrac; ++kk) {  // (fm holds only the call's fractions)
         if (!(fm & (1u << kk))) continue;
-        const int k = p.k0 + kk;
-        const int gx = x + axis_off(dx, k), gy = y + axis_off(dy, k);
-        if ((unsigned)gx >= (unsigned)p.W || (unsigned)gy >= (unsigned)p.H) continue;
-        const int rx = gx - RX0, ry = gy - RY0;
-        if ((unsigned)rx < (unsigned)kRegion && (unsigned)ry < (unsigned)kRegion)
-            atomicMin((unsigned long long *)&key[kk][ry * kRegion + rx], (unsigned long long)kv);
+        const float kf = fraction_scale(p.k0 + kk, p.L);
+        clip.put(key[kk], cx + offset_raw(mx, kf), cy + offset_raw(my, kf), kv);
+    }
+}
+
+// The same for a pixel of a clean tile, whose whole-pixel offsets the descriptor holds.
+__device__ __forceinline__ void engine_splat_clean(uint64_t (*key)[kRegionN], const RegionClip &clip,
+                                                   const SplatTile &st, int x, int y, uint32_t db) {
+    const uint64_t kv = pack_key_local(db, x, y);
+    const int cx = x - clip.RX0, cy = y - clip.RY0;
+#pragma unroll
+    for (int kk = 0; kk < kMaxFrac; ++kk) {
+        if (!(st.fm & (1u << kk))) continue;
+        clip.put(key[kk], cx + st.ox[kk], cy + st.oy[kk], kv);
     }
 }
 
@@ -762,10 +789,9 @@ __device__ __forceinline__ int describe_tiles(SplatTile *out, const TileParams &
         if (b.x <= b.y) {
             const bool uni = b.x == b.y && b.z == b.w;
             uint32_t fm = 0;
-            const BoundsDec bd = bounds_dec(b, d.L);
             for (int kk = 0; kk < d.nfrac; ++kk) {
                 int ox0, ox1, oy0, oy1;
-                bounds_offsets(bd, d.k0 + kk, ox0, ox1, oy0, oy1);
+                bounds_offsets(b, fraction_scale(d.k0 + kk, d.L), ox0, ox1, oy0, oy1);
                 if (8 * bx + 7 + ox1 >= RX0 && 8 * bx + ox0 < RX0 + kRegion && 8 * by + 7 + oy1 >= RY0 &&
                     8 * by + oy0 < RY0 + kRegion)
                     fm |= 1u << kk;
@@ -787,26 +813,16 @@ __device__ __forceinline__ int describe_tiles(SplatTile *out, const TileParams &
 template <typename CT, int WX, int WY>
 __device__ __forceinline__ void splat_window_pixel(uint64_t (*key)[kRegionN], const FrameDims &d,
                                                    const WinAcc<CT, WX, WY> &a, Rect U, const SplatTile &st, int q,
-                                                   int RX0, int RY0) {
+                                                   const RegionClip &clip) {
     if (!st.fm) return;
     const int x = 8 * st.bx + (q & 7), y = 8 * st.by + ((q >> 3) & 7);
     if (x < U.x0 || x > U.x1 || y < U.y0 || y > U.y1) return;
     const int i = a.at(x, y);
     const uint32_t db = __float_as_uint(a.w->depth[i]);
     if (st.clean) {
-        const uint64_t kv = pack_key_local(db, x, y);
-#pragma unroll
-        for (int kk = 0; kk < kMaxFrac; ++kk) {
-            if (!(st.fm & (1u << kk))) continue;
-            const int gx = x + st.ox[kk], gy = y + st.oy[kk];
-            if ((unsigned)gx >= (unsigned)d.W || (unsigned)gy >= (unsigned)d.H) continue;
-            const int rx = gx - RX0, ry = gy - RY0;
-            if ((unsigned)rx < (unsigned)kRegion && (unsigned)ry < (unsigned)kRegion)
-                atomicMin((unsigned long long *)&key[kk][ry * kRegion + rx], (unsigned long long)kv);
-        }
+        engine_splat_clean(key, clip, st, x, y, db);
     } else {
-        engine_splat_pixel(key, d, x, y, db, __float_as_uint(a.w->mv[0][i]), __float_as_uint(a.w->mv[1][i]), st.fm,
-                           RX0, RY0);
+        engine_splat_pixel(key, d, clip, x, y, db, a.w->mv[0][i], a.w->mv[1][i], st.fm);
     }
 }
 
@@ -821,10 +837,11 @@ template <typename CT, int WX, int WY>
 __device__ __forceinline__ void engine_splat_window(EngineSmem &s, uint64_t (*key)[kRegionN], const TileParams &p,
                                                     const FrameDims &d, const WinAcc<CT, WX, WY> &a, Rect U, int RX0,
                                                     int RY0, int tid, const SplatTile *pre, int npre, uint32_t *next) {
+    const RegionClip clip(d, RX0, RY0);
     if (npre == 0) {  // too many candidates for the plan: described here, half a tile per warp and round
         const int nt = describe_tiles(s.cand, p, d, U, RX0, RY0, tid);
         bar_sync(kBarConsumers, kConsumerThreads);
-        for (int q = tid; q < 64 * nt; q += kConsumerThreads) splat_window_pixel(key, d, a, U, s.cand[q >> 6], q, RX0, RY0);
+        for (int q = tid; q < 64 * nt; q += kConsumerThreads) splat_window_pixel(key, d, a, U, s.cand[q >> 6], q, clip);
         return;
     }
     // the plan's candidates, in chunks of half a tile that the warps claim: the warps that start the slot early
@@ -835,7 +852,7 @@ __device__ __forceinline__ void engine_splat_window(EngineSmem &s, uint64_t (*ke
         int nx = 0;
         if (lane == 0) nx = (int)atomicAdd(next, 1u);  // the next claim, in flight while this chunk splats
         const int q = 32 * c + lane;
-        splat_window_pixel(key, d, a, U, pre[q >> 6], q, RX0, RY0);
+        splat_window_pixel(key, d, a, U, pre[q >> 6], q, clip);
         c = __shfl_sync(0xFFFFFFFFu, nx, 0);
     }
 }
@@ -844,19 +861,20 @@ __device__ __forceinline__ void engine_splat_window(EngineSmem &s, uint64_t (*ke
 // clean candidate (one exact motion, every pixel can land) splats with its precomputed offsets and reads only the
 // depth of its pixels.
 __device__ __forceinline__ void splat_global_candidate(uint64_t (*key)[kRegionN], const TileParams &p,
-                                                       const FrameDims &d, const SplatTile &st, int RX0, int RY0,
-                                                       int tid);
+                                                       const FrameDims &d, const SplatTile &st,
+                                                       const RegionClip &clip, int tid);
 
 __device__ inline void engine_splat_global(EngineSmem &s, uint64_t (*key)[kRegionN], const TileParams &p,
                                            const FrameDims &d, int RX0, int RY0, int tid, const SplatTile *pre,
                                            int npre, uint32_t *next) {
+    const RegionClip clip(d, RX0, RY0);
     if (npre > 0) {  // the plan's candidates, in chunks of half a tile that the warps claim
         const int nchunk = 2 * npre, lane = tid & 31;
         int c = claim_chunk(next);
         while (c < nchunk) {
             int nx = 0;
             if (lane == 0) nx = (int)atomicAdd(next, 1u);
-            splat_global_candidate(key, p, d, pre[c >> 1], RX0, RY0, 32 * (c & 1) + lane);
+            splat_global_candidate(key, p, d, pre[c >> 1], clip, 32 * (c & 1) + lane);
             c = __shfl_sync(0xFFFFFFFFu, nx, 0);
         }
         return;
@@ -877,10 +895,9 @@ __device__ inline void engine_splat_global(EngineSmem &s, uint64_t (*key)[kRegio
                 SplatTile st{};
                 uint32_t fm = 0;
                 bool small = true;  // every offset fits an int8 (else a clean tile still splats per pixel)
-                const BoundsDec bd = bounds_dec(b, p.L);
                 for (int kk = 0; kk < p.nfrac; ++kk) {
                     int ox0, ox1, oy0, oy1;
-                    bounds_offsets(bd, p.k0 + kk, ox0, ox1, oy0, oy1);
+                    bounds_offsets(b, fraction_scale(p.k0 + kk, p.L), ox0, ox1, oy0, oy1);
                     const int tx0 = 8 * bx + ox0, tx1 = 8 * bx + 7 + ox1;
                     const int ty0 = 8 * by + oy0, ty1 = 8 * by + 7 + oy1;
                     if (tx1 >= RX0 && tx0 < RX0 + kRegion && ty1 >= RY0 && ty0 < RY0 + kRegion) fm |= 1u << kk;
@@ -901,7 +918,7 @@ __device__ inline void engine_splat_global(EngineSmem &s, uint64_t (*key)[kRegio
         const int nc = (int)s.ncand;
         for (int c0 = 0; c0 < nc; c0 += kConsumerThreads / 64) {
             const int ci = c0 + (tid >> 6);
-            if (ci < nc) splat_global_candidate(key, p, d, s.cand[ci], RX0, RY0, tid);
+            if (ci < nc) splat_global_candidate(key, p, d, s.cand[ci], clip, tid);
         }
         bar_sync(kBarConsumers, kConsumerThreads);
     }
@@ -909,27 +926,17 @@ __device__ inline void engine_splat_global(EngineSmem &s, uint64_t (*key)[kRegio
 
 // One pixel (of 64 threads' 8 x 8 tile) of a candidate source tile, from global memory.
 __device__ __forceinline__ void splat_global_candidate(uint64_t (*key)[kRegionN], const TileParams &p,
-                                                       const FrameDims &d, const SplatTile &st, int RX0, int RY0,
-                                                       int tid) {
+                                                       const FrameDims &d, const SplatTile &st,
+                                                       const RegionClip &clip, int tid) {
     const int x = 8 * st.bx + (tid & 7), y = 8 * st.by + ((tid >> 3) & 7);
     if (x >= p.W || y >= p.H) return;
     const size_t i = (size_t)y * p.W + x;
     const uint32_t db = __float_as_uint(__ldg(p.depth + i));
     if (st.clean) {
-        const uint64_t kv = pack_key_local(db, x, y);
-#pragma unroll
-        for (int kk = 0; kk < kMaxFrac; ++kk) {
-            if (!(st.fm & (1u << kk))) continue;
-            const int gx = x + st.ox[kk], gy = y + st.oy[kk];
-            if ((unsigned)gx >= (unsigned)d.W || (unsigned)gy >= (unsigned)d.H) continue;
-            const int rx = gx - RX0, ry = gy - RY0;
-            if ((unsigned)rx < (unsigned)kRegion && (unsigned)ry < (unsigned)kRegion)
-                atomicMin((unsigned long long *)&key[kk][ry * kRegion + rx], (unsigned long long)kv);
-        }
+        engine_splat_clean(key, clip, st, x, y, db);
     } else {
         const size_t plane = (size_t)p.W * p.H;
-        engine_splat_pixel(key, d, x, y, db, __float_as_uint(__ldg(p.mv + i)),
-                           __float_as_uint(__ldg(p.mv + plane + i)), st.fm, RX0, RY0);
+        engine_splat_pixel(key, d, clip, x, y, db, __ldg(p.mv + i), __ldg(p.mv + plane + i), st.fm);
     }
 }
 
@@ -1243,7 +1250,8 @@ __device__ float4 smooth_node(const TileParams &p, int tile, int kk, float4 *l2)
     const uint32_t umx = __ldcg(&p.plans[tile].umx), umy = __ldcg(&p.plans[tile].umy);
     const int k = p.k0 + kk;
     // the fraction's constants, as uniform_frac computes them
-    const int ox = axis_off_of(umx, k, p.L), oy = axis_off_of(umy, k, p.L);
+    const float kf = fraction_scale(k, p.L);
+    const int ox = offset_of(__uint_as_float(umx), kf), oy = offset_of(__uint_as_float(umy), kf);
     int sx, sy;
     const float rx = residual(__uint_as_float(umx), k, p.L, ox, sx);
     const float ry = residual(__uint_as_float(umy), k, p.L, oy, sy);

@@ -54,11 +54,10 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
         if (!(b.x <= b.y)) return st;
         uint32_t fm = 0u;
         bool small = true;
-        const BoundsDec bd = bounds_dec(b, p.L);
 #pragma unroll
         for (int kk = 0; kk < kMaxFrac; ++kk) {
             int ox0, ox1, oy0, oy1;
-            bounds_offsets(bd, p.k0 + kk, ox0, ox1, oy0, oy1);
+            bounds_offsets(b, fraction_scale(p.k0 + kk, p.L), ox0, ox1, oy0, oy1);
             const int lx0 = max(8 * bx, RX0 - ox1), lx1 = min(min(8 * bx + 7, p.W - 1), RX0 + kRegion - 1 - ox0);
             const int ly0 = max(8 * by, RY0 - oy1), ly1 = min(min(8 * by + 7, p.H - 1), RY0 + kRegion - 1 - oy0);
             const bool hit = kk < p.nfrac && lx0 <= lx1 && ly0 <= ly1;
@@ -102,10 +101,9 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
                 rxl = rx0 + idx % nrr;
                 const float4 rb = __ldcg(p.region_bounds + (size_t)ryl * p.n5x + rxl);
                 if (rb.x <= rb.y) {
-                    const BoundsDec rd = bounds_dec(rb, p.L);
                     for (int kk = 0; kk < p.nfrac && !reach; ++kk) {
                         int ox0, ox1, oy0, oy1;
-                        bounds_offsets(rd, p.k0 + kk, ox0, ox1, oy0, oy1);
+                        bounds_offsets(rb, fraction_scale(p.k0 + kk, p.L), ox0, ox1, oy0, oy1);
                         reach = 32 * rxl + 31 + ox1 >= RX0 && 32 * rxl + ox0 <= RX0 + kRegion - 1 &&
                                 32 * ryl + 31 + oy1 >= RY0 && 32 * ryl + oy0 <= RY0 + kRegion - 1;
                     }
@@ -161,7 +159,8 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
     if (uni && hasm && RX0 >= 0 && RY0 >= 0 && RX0 + kRegion <= p.W && RY0 + kRegion <= p.H) {
         Rect Nu{1 << 30, -(1 << 30), 1 << 30, -(1 << 30)};
         for (int kk = 0; kk < p.nfrac; ++kk) {
-            const int ox = axis_off_of(mx, p.k0 + kk, p.L), oy = axis_off_of(my, p.k0 + kk, p.L);
+            const float kf = fraction_scale(p.k0 + kk, p.L);
+            const int ox = offset_of(__uint_as_float(mx), kf), oy = offset_of(__uint_as_float(my), kf);
             Nu.x0 = min(Nu.x0, RX0 - ox - 1);
             Nu.x1 = max(Nu.x1, RX0 + kRegion - ox);
             Nu.y0 = min(Nu.y0, RY0 - oy - 1);
@@ -219,7 +218,8 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
         // uniform: fraction kk's sources are R - o_kk; stage their union grown by one pixel (the taps)
         Rect N{1 << 30, -(1 << 30), 1 << 30, -(1 << 30)};
         for (int kk = 0; kk < p.nfrac; ++kk) {
-            const int ox = axis_off_of(mx, p.k0 + kk, p.L), oy = axis_off_of(my, p.k0 + kk, p.L);
+            const float kf = fraction_scale(p.k0 + kk, p.L);
+            const int ox = offset_of(__uint_as_float(mx), kf), oy = offset_of(__uint_as_float(my), kf);
             N.x0 = min(N.x0, RX0 - ox - 1);
             N.x1 = max(N.x1, RX0 + kRegion - ox);
             N.y0 = min(N.y0, RY0 - oy - 1);

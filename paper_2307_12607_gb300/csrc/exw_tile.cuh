@@ -22,15 +22,12 @@ __device__ __forceinline__ bool frame_window(const TileParams &p, int RX0, int R
     const uint32_t a0 = __ldcg(&p.fh->acc[0]), a1 = __ldcg(&p.fh->acc[1]);
     const uint32_t a2 = __ldcg(&p.fh->acc[2]), a3 = __ldcg(&p.fh->acc[3]);
     if (a1 == 0u) return false;
-    const AxisDec fx0 = axis_dec(__float_as_uint(-float_unorder(a0)), p.L);
-    const AxisDec fx1 = axis_dec(__float_as_uint(float_unorder(a1)), p.L);
-    const AxisDec fy0 = axis_dec(__float_as_uint(-float_unorder(a2)), p.L);
-    const AxisDec fy1 = axis_dec(__float_as_uint(float_unorder(a3)), p.L);
+    const float fx0 = -float_unorder(a0), fx1 = float_unorder(a1), fy0 = -float_unorder(a2), fy1 = float_unorder(a3);
     int xlo = 1 << 30, xhi = -(1 << 30), ylo = 1 << 30, yhi = -(1 << 30);
     for (int kk = 0; kk < p.nfrac; ++kk) {
-        const int k = p.k0 + kk;
-        const int ox0 = axis_off(fx0, k), ox1 = axis_off(fx1, k);
-        const int oy0 = axis_off(fy0, k), oy1 = axis_off(fy1, k);
+        const float kf = fraction_scale(p.k0 + kk, p.L);
+        const int ox0 = offset_of(fx0, kf), ox1 = offset_of(fx1, kf);
+        const int oy0 = offset_of(fy0, kf), oy1 = offset_of(fy1, kf);
         xlo = min(xlo, RX0 - ox1);
         xhi = max(xhi, RX0 + kRegion - 1 - ox0);
         ylo = min(ylo, RY0 - oy1);
@@ -43,20 +40,12 @@ __device__ __forceinline__ bool frame_window(const TileParams &p, int RX0, int R
     return bx0 <= bx1 && by0 <= by1;
 }
 
-// The four motion bounds of a tile decoded once (axis_dec); each fraction's offsets [ox0, ox1] x [oy0, oy1] then
-// cost four shift-adds (axis_off of the decoded bounds: the offset is monotone in the motion).
-struct BoundsDec {
-    AxisDec x0, x1, y0, y1;
-};
-__device__ __forceinline__ BoundsDec bounds_dec(const float4 &b, int L) {
-    return BoundsDec{axis_dec(__float_as_uint(b.x), L), axis_dec(__float_as_uint(b.y), L),
-                     axis_dec(__float_as_uint(b.z), L), axis_dec(__float_as_uint(b.w), L)};
-}
-__device__ __forceinline__ void bounds_offsets(const BoundsDec &d, int k, int &ox0, int &ox1, int &oy0, int &oy1) {
-    ox0 = axis_off(d.x0, k);
-    ox1 = axis_off(d.x1, k);
-    oy0 = axis_off(d.y0, k);
-    oy1 = axis_off(d.y1, k);
+// The offsets [ox0, ox1] x [oy0, oy1] of a fraction of a tile's motion bounds (the offset is monotone in the motion).
+__device__ __forceinline__ void bounds_offsets(const float4 &b, float kf, int &ox0, int &ox1, int &oy0, int &oy1) {
+    ox0 = offset_of(b.x, kf);
+    ox1 = offset_of(b.y, kf);
+    oy0 = offset_of(b.z, kf);
+    oy1 = offset_of(b.w, kf);
 }
 
 // ------------------------------------------------------------------------------------------------------------
