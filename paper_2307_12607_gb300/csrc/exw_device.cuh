@@ -197,6 +197,18 @@ __device__ __forceinline__ float4 mean4(float4 c0, float4 c1, float4 c2, float4 
     return make_float4(__fmul_rn(a0, inv), __fmul_rn(a1, inv), __fmul_rn(a2, inv), 1.0f);
 }
 
+// The same where every .w is 0 or 1 and an invalid node's colour is 0 (all but the coarse levels): adding the zeros of
+// the invalid children changes no bit, so nothing is selected.
+// A third fewer instructions a node: a recursive chain at 1080p FP32 147.7 -> 139.6 us, splat + warp + fill at 720p FP16
+// 29.2 -> 27.4.
+__device__ __forceinline__ float4 mean4_01(float4 c0, float4 c1, float4 c2, float4 c3) {
+    const float n = (c0.w + c1.w) + (c2.w + c3.w);
+    const float inv = n == 1.0f ? 1.0f : n == 2.0f ? 0.5f : n == 3.0f ? (1.0f / 3.0f) : 0.25f;
+    return make_float4(__fmul_rn(__fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(0.0f, c0.x), c1.x), c2.x), c3.x), inv),
+                       __fmul_rn(__fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(0.0f, c0.y), c1.y), c2.y), c3.y), inv),
+                       __fmul_rn(__fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(0.0f, c0.z), c1.z), c2.z), c3.z), inv), fminf(n, 1.0f));
+}
+
 __device__ __forceinline__ float4 shfl4_xor(float4 v, int m) {
     return make_float4(__shfl_xor_sync(0xFFFFFFFFu, v.x, m), __shfl_xor_sync(0xFFFFFFFFu, v.y, m),
                        __shfl_xor_sync(0xFFFFFFFFu, v.z, m), __shfl_xor_sync(0xFFFFFFFFu, v.w, m));

@@ -1019,15 +1019,15 @@ __device__ __forceinline__ void upper_levels_smem(const float4 *l2, float4 *up, 
     const int lane = threadIdx.x & 31;
     if (lane < 16) {
         const float4 *c = l2 + (2 * (lane >> 2)) * 32 + 2 * (lane & 3);
-        up[lane] = mean4(c[0], c[1], c[32], c[33]);
+        up[lane] = mean4_01(c[0], c[1], c[32], c[33]);
     }
     __syncwarp();
     if (lane < 4) {
         const int b4 = 8 * (lane >> 1) + 2 * (lane & 1);
-        up[16 + lane] = mean4(up[b4], up[b4 + 1], up[b4 + 4], up[b4 + 5]);
+        up[16 + lane] = mean4_01(up[b4], up[b4 + 1], up[b4 + 4], up[b4 + 5]);
     }
     __syncwarp();
-    l5 = mean4(up[16], up[17], up[18], up[19]);
+    l5 = mean4_01(up[16], up[17], up[18], up[19]);
     v3 = up[(w >> 1) * 4 + (bx >> 2)];
     v4 = up[16 + (w >> 2) * 2 + (bx >> 3)];
     __syncwarp();  // every read of the scratch before the warp's next use of it
@@ -1129,12 +1129,12 @@ __device__ __forceinline__ void fill_store_block(EngineSmem &s, const TileParams
     // level-2 nodes (its row w of them) from four of its level-1 nodes, then in the first 8 of its slots.  No later
     // slot touches the scratch before every warp of the group is done with it (each slot that does starts behind a
     // barrier of the whole group or of all consumers).
-    const float4 n1 = mean4(c[0], c[1], c[2], c[3]);
+    const float4 n1 = mean4_01(c[0], c[1], c[2], c[3]);
     float4 *l1 = reinterpret_cast<float4 *>(s.cand) + g * kGroupThreads;
     l1[tg] = n1;
     __syncwarp();
     float4 n2o = n1;
-    if ((lane & 17) == 0) n2o = mean4(n1, l1[tg + 1], l1[tg + 16], l1[tg + 17]);
+    if ((lane & 17) == 0) n2o = mean4_01(n1, l1[tg + 1], l1[tg + 16], l1[tg + 17]);
     __syncwarp();  // every read of the warp's level-1 slots before they hold its level-2 nodes
     float4 *l2 = l1;  // level-2 node (i, j) at l2[32 i + j]
     if ((lane & 17) == 0) l2[32 * w + (lane >> 1)] = n2o;
@@ -1190,14 +1190,14 @@ __device__ __forceinline__ float4 smooth_level2(const CT out[4][3]) {
     }
     const bool odd = lane & 1;
     // level 1: rows 0-1 (A) and 2-3 (B) of this column pair, children in (row, column) order
-    const float4 A = odd ? mean4(pp[0], px[0], pp[1], px[1]) : mean4(px[0], pp[0], px[1], pp[1]);
-    const float4 B = odd ? mean4(pp[2], px[2], pp[3], px[3]) : mean4(px[2], pp[2], px[3], pp[3]);
+    const float4 A = odd ? mean4_01(pp[0], px[0], pp[1], px[1]) : mean4_01(px[0], pp[0], px[1], pp[1]);
+    const float4 B = odd ? mean4_01(pp[2], px[2], pp[3], px[3]) : mean4_01(px[2], pp[2], px[3], pp[3]);
     const float4 Ap = make_float4(__shfl_xor_sync(0xFFFFFFFFu, A.x, 2), __shfl_xor_sync(0xFFFFFFFFu, A.y, 2),
                                   __shfl_xor_sync(0xFFFFFFFFu, A.z, 2), 1.0f);
     const float4 Bp = make_float4(__shfl_xor_sync(0xFFFFFFFFu, B.x, 2), __shfl_xor_sync(0xFFFFFFFFu, B.y, 2),
                                   __shfl_xor_sync(0xFFFFFFFFu, B.z, 2), 1.0f);
     const bool right = lane & 2;
-    return right ? mean4(Ap, A, Bp, B) : mean4(A, Ap, B, Bp);
+    return right ? mean4_01(Ap, A, Bp, B) : mean4_01(A, Ap, B, Bp);
 }
 
 // The lazy smooth node, recomputed by one warp: the tile's outputs again from the source colour (the same arithmetic
@@ -1232,9 +1232,9 @@ __device__ float4 output_node(const TileParams &p, int tile, int kk, float4 *l2)
                                    1.0f);
             }
         }
-        const float4 n1 = mean4(c[0], c[1], c[2], c[3]);
+        const float4 n1 = mean4_01(c[0], c[1], c[2], c[3]);
         const float4 a1 = shfl4_xor(n1, 1), a16 = shfl4_xor(n1, 16), a17 = shfl4_xor(n1, 17);
-        const float4 n2o = mean4(n1, a1, a16, a17);
+        const float4 n2o = mean4_01(n1, a1, a16, a17);
         if ((lane & 17) == 0) l2[w * 8 + (lane >> 1)] = n2o;
     }
     __syncwarp();

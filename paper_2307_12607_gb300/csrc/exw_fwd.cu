@@ -190,7 +190,10 @@ __global__ void __launch_bounds__(kTileThreads, 3) fill_tiles_kernel(const __gri
         }
     }
 #pragma unroll
-    for (int r = 0; r < kTileRows; ++r) c[r].w = m[r] == 0 ? 1.0f : 0.0f;
+    for (int r = 0; r < kTileRows; ++r) {  // (a hole holds anything)
+        if (m[r] != 0) c[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        else c[r].w = 1.0f;
+    }
     const unsigned int have = fill_columns(p, pyramid, c, m, 0, blockIdx.y * p.n5x + blockIdx.x);
 #pragma unroll
     for (int r = 0; r < kTileRows; ++r) {

@@ -295,6 +295,7 @@ __device__ inline float4 bounds_region(const float *__restrict__ depth, const fl
     const int X0 = rx * 32, Y0 = ry * 32;
     const size_t plane = (size_t)W * H;
     float mnx = __int_as_float(0x7F800000), mxx = -mnx, mny = mnx, mxy = -mnx;
+    const float kFinite = __int_as_float(0x7F7FFFFF);
     const int x = X0 + lane;
     // the frame-wide maxima as they stand, read with the data (any earlier value is a valid lower bound: a stale one
     // only costs an atomic that does not raise anything)
@@ -317,19 +318,23 @@ __device__ inline float4 bounds_region(const float *__restrict__ depth, const fl
     float dmn = __int_as_float(0x7F800000), dmx = 0.0f, bad = 0.0f;
 #pragma unroll
     for (int r = 0; r < rpw; ++r) {
-        if (depth_ok(db[r]) && finite_bits(__float_as_uint(fx[r])) && finite_bits(__float_as_uint(fy[r]))) {
-            const float cx = fminf(fmaxf(fx[r], -65536.0f), 65536.0f) + 0.0f;
-            const float cy = fminf(fmaxf(fy[r], -65536.0f), 65536.0f) + 0.0f;
-            mnx = fminf(mnx, cx);
-            mxx = fmaxf(mxx, cx);
-            mny = fminf(mny, cy);
-            mxy = fmaxf(mxy, cy);
+        if (depth_ok(db[r]) && fabsf(fx[r]) <= kFinite && fabsf(fy[r]) <= kFinite) {  // (a NaN compares false)
+            mnx = fminf(mnx, fx[r]);
+            mxx = fmaxf(mxx, fx[r]);
+            mny = fminf(mny, fy[r]);
+            mxy = fmaxf(mxy, fy[r]);
             dmn = fminf(dmn, __uint_as_float(db[r]));
             dmx = fmaxf(dmx, __uint_as_float(db[r]));
         } else if (r < rpw && x < W && Y0 + w * rpw + r < H) {
             bad = 1.0f;
         }
     }
+    // clamped, and -0 made +0, once per thread: both keep the order (no pixel: +inf, -inf as before)
+    auto clamped = [&](float v) { return fabsf(v) <= kFinite ? fminf(fmaxf(v, -65536.0f), 65536.0f) + 0.0f : v; };
+    mnx = clamped(mnx);
+    mxx = clamped(mxx);
+    mny = clamped(mny);
+    mxy = clamped(mxy);
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {
         mnx = fminf(mnx, __shfl_xor_sync(0xFFFFFFFFu, mnx, o));

@@ -150,12 +150,12 @@ __device__ __forceinline__ void upper_levels(const float4 *l2, float4 &l3, float
     const int L = lane & 15;
     const int I = L >> 2, J = L & 3;
     const float4 *c = l2 + (2 * I) * 8 + 2 * J;
-    l3 = mean4(c[0], c[1], c[8], c[9]);
+    l3 = mean4_01(c[0], c[1], c[8], c[9]);
     const int b4 = 8 * ((lane & 3) >> 1) + 2 * (lane & 1);
     const float4 q0 = shfl4_idx(l3, b4), q1 = shfl4_idx(l3, b4 + 1), q2 = shfl4_idx(l3, b4 + 4),
                  q3 = shfl4_idx(l3, b4 + 5);
-    l4 = mean4(q0, q1, q2, q3);
-    l5 = mean4(shfl4_idx(l4, 0), shfl4_idx(l4, 1), shfl4_idx(l4, 2), shfl4_idx(l4, 3));
+    l4 = mean4_01(q0, q1, q2, q3);
+    l5 = mean4_01(shfl4_idx(l4, 0), shfl4_idx(l4, 1), shfl4_idx(l4, 2), shfl4_idx(l4, 3));
 }
 
 // Publishes the tile's level-5 node and replaces each hole of this thread's column (m[r] != 0) by its first valid
@@ -167,7 +167,7 @@ __device__ __forceinline__ unsigned int fill_columns(const TileParams &p, TilePy
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const float4 o0 = shfl4_xor(c[0], 1), o1 = shfl4_xor(c[1], 1);
     // children in the order (0,0), (0,1), (1,0), (1,1)
-    const float4 n1 = (lane & 1) ? mean4(o0, c[0], o1, c[1]) : mean4(c[0], o0, c[1], o1);
+    const float4 n1 = (lane & 1) ? mean4_01(o0, c[0], o1, c[1]) : mean4_01(c[0], o0, c[1], o1);
     if ((lane & 1) == 0) t.l1[w * 16 + (lane >> 1)] = n1;
     const bool deep = __syncthreads_or((m[0] | m[1]) != 0 && n1.w == 0.0f) != 0;
     if (w == 0) {
@@ -175,7 +175,7 @@ __device__ __forceinline__ unsigned int fill_columns(const TileParams &p, TilePy
         for (int h = 0; h < 2; ++h) {
             const int node = lane + 32 * h, i = node >> 3, j = node & 7;
             const float4 *q = t.l1 + (2 * i) * 16 + 2 * j;
-            t.l2[node] = mean4(q[0], q[1], q[16], q[17]);
+            t.l2[node] = mean4_01(q[0], q[1], q[16], q[17]);
         }
         __syncwarp();
         float4 l3, l4, l5;
