@@ -120,8 +120,8 @@ static bool build_params(EngineParams *ep, const EngineSpec *specs, int first, i
         p.W = f.W;
         p.H = f.H;
         p.nfrac = nfrac;
-        p.L = 2;
-        p.k0 = 1;
+        p.L = kEngineL;
+        p.k0 = kEngineK0;
         for (int j = 0; j < nfrac; ++j) {
             p.out_color[j] = sp.out[j].color;
             p.out_mask[j] = sp.out[j].mask;

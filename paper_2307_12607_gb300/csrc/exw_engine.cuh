@@ -96,9 +96,9 @@ constexpr uint32_t kTapX = 1u, kTapY = 2u, kMirX = 4u, kMirY = 8u;
 // The scalars of a stream the per-pixel code needs, held in registers for a whole tile (the slot's parameters sit
 // in shared memory, and every barrier would otherwise reload them).
 struct FrameDims {
-    int W, H, L, k0, nfrac;
+    int W, H, nfrac;
 };
-__device__ __forceinline__ FrameDims dims_of(const TileParams &p) { return FrameDims{p.W, p.H, p.L, p.k0, p.nfrac}; }
+__device__ __forceinline__ FrameDims dims_of(const TileParams &p) { return FrameDims{p.W, p.H, p.nfrac}; }
 
 // What the producer hands the consumers with each buffer.
 struct alignas(16) TileSlot {
@@ -202,12 +202,12 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t *mbar, uint32_t pari
 // writes inv[j]).
 __device__ __forceinline__ void uniform_frac(UniformFrac &u, const TileParams &p, uint32_t umx, uint32_t umy, int kk,
                                              int j) {
-    const int k = p.k0 + kk;
-    const float kf = fraction_scale(k, p.L);
+    const int k = kEngineK0 + kk;
+    const float kf = engine_scale(kk);
     const int ox = offset_of(__uint_as_float(umx), kf), oy = offset_of(__uint_as_float(umy), kf);
     int sx, sy;
-    const float rx = residual(__uint_as_float(umx), k, p.L, ox, sx);
-    const float ry = residual(__uint_as_float(umy), k, p.L, oy, sy);
+    const float rx = residual(__uint_as_float(umx), k, kEngineL, ox, sx);
+    const float ry = residual(__uint_as_float(umy), k, kEngineL, oy, sy);
     const float wx1 = fabsf(rx), wy1 = fabsf(ry);
     const float wx0 = 1.0f - wx1, wy0 = 1.0f - wy1;
     const float W00 = __fmul_rn(wx0, wy0), W10 = __fmul_rn(wx1, wy0), W01 = __fmul_rn(wx0, wy1),
@@ -741,7 +741,7 @@ __device__ __forceinline__ void engine_splat_pixel(uint64_t (*key)[kRegionN], co
 #pragma unroll
     for (int kk = 0; kk < kMaxFrac; ++kk) {  // (fm holds only the call's fractions)
         if (!(fm & (1u << kk))) continue;
-        const float kf = fraction_scale(p.k0 + kk, p.L);
+        const float kf = engine_scale(kk);
         clip.put(key[kk], cx + offset_raw(mx, kf), cy + offset_raw(my, kf), kv);
     }
 }
@@ -791,7 +791,7 @@ __device__ __forceinline__ int describe_tiles(SplatTile *out, const TileParams &
             uint32_t fm = 0;
             for (int kk = 0; kk < d.nfrac; ++kk) {
                 int ox0, ox1, oy0, oy1;
-                bounds_offsets(b, fraction_scale(d.k0 + kk, d.L), ox0, ox1, oy0, oy1);
+                bounds_offsets(b, engine_scale(kk), ox0, ox1, oy0, oy1);
                 if (8 * bx + 7 + ox1 >= RX0 && 8 * bx + ox0 < RX0 + kRegion && 8 * by + 7 + oy1 >= RY0 &&
                     8 * by + oy0 < RY0 + kRegion)
                     fm |= 1u << kk;
@@ -897,7 +897,7 @@ __device__ inline void engine_splat_global(EngineSmem &s, uint64_t (*key)[kRegio
                 bool small = true;  // every offset fits an int8 (else a clean tile still splats per pixel)
                 for (int kk = 0; kk < p.nfrac; ++kk) {
                     int ox0, ox1, oy0, oy1;
-                    bounds_offsets(b, fraction_scale(p.k0 + kk, p.L), ox0, ox1, oy0, oy1);
+                    bounds_offsets(b, engine_scale(kk), ox0, ox1, oy0, oy1);
                     const int tx0 = 8 * bx + ox0, tx1 = 8 * bx + 7 + ox1;
                     const int ty0 = 8 * by + oy0, ty1 = 8 * by + 7 + oy1;
                     if (tx1 >= RX0 && tx0 < RX0 + kRegion && ty1 >= RY0 && ty0 < RY0 + kRegion) fm |= 1u << kk;
@@ -959,8 +959,8 @@ __device__ __forceinline__ void gather_pixel(const uint32_t *kw, const Acc &a, c
     }
     const auto i00 = a.at(px, py);
     int sx, sy;
-    const float rx = residual(a.mx(i00), k, p.L, gx - px, sx);
-    const float ry = residual(a.my(i00), k, p.L, gy - py, sy);
+    const float rx = residual(a.mx(i00), k, kEngineL, gx - px, sx);
+    const float ry = residual(a.my(i00), k, kEngineL, gy - py, sy);
     const float wx1 = fabsf(rx), wy1 = fabsf(ry);
     const float wx0 = 1.0f - wx1, wy0 = 1.0f - wy1;
     const bool ex = sx != 0 && (unsigned)(px + sx) < (unsigned)p.W;
@@ -1248,13 +1248,13 @@ template <typename CT>
 __device__ float4 smooth_node(const TileParams &p, int tile, int kk, float4 *l2) {
     const int lane = threadIdx.x & 31;
     const uint32_t umx = __ldcg(&p.plans[tile].umx), umy = __ldcg(&p.plans[tile].umy);
-    const int k = p.k0 + kk;
+    const int k = kEngineK0 + kk;
     // the fraction's constants, as uniform_frac computes them
-    const float kf = fraction_scale(k, p.L);
+    const float kf = engine_scale(kk);
     const int ox = offset_of(__uint_as_float(umx), kf), oy = offset_of(__uint_as_float(umy), kf);
     int sx, sy;
-    const float rx = residual(__uint_as_float(umx), k, p.L, ox, sx);
-    const float ry = residual(__uint_as_float(umy), k, p.L, oy, sy);
+    const float rx = residual(__uint_as_float(umx), k, kEngineL, ox, sx);
+    const float ry = residual(__uint_as_float(umy), k, kEngineL, oy, sy);
     const float wx1 = fabsf(rx), wy1 = fabsf(ry);
     const float wx0 = 1.0f - wx1, wy0 = 1.0f - wy1;
     const float W00 = __fmul_rn(wx0, wy0), W10 = __fmul_rn(wx1, wy0), W01 = __fmul_rn(wx0, wy1),
@@ -1502,7 +1502,7 @@ __device__ __forceinline__ void tile_group(EngineSmem &s, const TileSlot &sl, co
     const int bx = tg & 15, by = tg >> 4;
     const int mode = sl.plan.mode, tile = sl.index, X0 = sl.X0, Y0 = sl.Y0;
     const int wx0 = sl.plan.wx0, wy0 = sl.plan.wy0;
-    const int kk = g, k = d.k0 + kk;
+    const int kk = g, k = kEngineK0 + kk;
     const int TX = X0 + 2 * bx, TY = Y0 + 2 * by;
     CT *oc = (CT *)p.out_color[kk];
     uint8_t *om = p.out_mask[kk];

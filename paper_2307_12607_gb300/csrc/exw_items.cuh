@@ -57,7 +57,7 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
 #pragma unroll
         for (int kk = 0; kk < kMaxFrac; ++kk) {
             int ox0, ox1, oy0, oy1;
-            bounds_offsets(b, fraction_scale(p.k0 + kk, p.L), ox0, ox1, oy0, oy1);
+            bounds_offsets(b, engine_scale(kk), ox0, ox1, oy0, oy1);
             const int lx0 = max(8 * bx, RX0 - ox1), lx1 = min(min(8 * bx + 7, p.W - 1), RX0 + kRegion - 1 - ox0);
             const int ly0 = max(8 * by, RY0 - oy1), ly1 = min(min(8 * by + 7, p.H - 1), RY0 + kRegion - 1 - oy0);
             const bool hit = kk < p.nfrac && lx0 <= lx1 && ly0 <= ly1;
@@ -103,7 +103,7 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
                 if (rb.x <= rb.y) {
                     for (int kk = 0; kk < p.nfrac && !reach; ++kk) {
                         int ox0, ox1, oy0, oy1;
-                        bounds_offsets(rb, fraction_scale(p.k0 + kk, p.L), ox0, ox1, oy0, oy1);
+                        bounds_offsets(rb, engine_scale(kk), ox0, ox1, oy0, oy1);
                         reach = 32 * rxl + 31 + ox1 >= RX0 && 32 * rxl + ox0 <= RX0 + kRegion - 1 &&
                                 32 * ryl + 31 + oy1 >= RY0 && 32 * ryl + oy0 <= RY0 + kRegion - 1;
                     }
@@ -159,7 +159,7 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
     if (uni && hasm && RX0 >= 0 && RY0 >= 0 && RX0 + kRegion <= p.W && RY0 + kRegion <= p.H) {
         Rect Nu{1 << 30, -(1 << 30), 1 << 30, -(1 << 30)};
         for (int kk = 0; kk < p.nfrac; ++kk) {
-            const float kf = fraction_scale(p.k0 + kk, p.L);
+            const float kf = engine_scale(kk);
             const int ox = offset_of(__uint_as_float(mx), kf), oy = offset_of(__uint_as_float(my), kf);
             Nu.x0 = min(Nu.x0, RX0 - ox - 1);
             Nu.x1 = max(Nu.x1, RX0 + kRegion - ox);
@@ -218,7 +218,7 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
         // uniform: fraction kk's sources are R - o_kk; stage their union grown by one pixel (the taps)
         Rect N{1 << 30, -(1 << 30), 1 << 30, -(1 << 30)};
         for (int kk = 0; kk < p.nfrac; ++kk) {
-            const float kf = fraction_scale(p.k0 + kk, p.L);
+            const float kf = engine_scale(kk);
             const int ox = offset_of(__uint_as_float(mx), kf), oy = offset_of(__uint_as_float(my), kf);
             N.x0 = min(N.x0, RX0 - ox - 1);
             N.x1 = max(N.x1, RX0 + kRegion - ox);
