@@ -10,6 +10,7 @@ Layouts (see include/exw.h): colour [3][H][W] float32/float16, depth [H][W] floa
 from __future__ import annotations
 
 import ctypes
+import struct
 
 import torch
 
@@ -30,8 +31,14 @@ class ExwError(RuntimeError):
         self.status = status
 
 
+_loaded = None
+
+
 def lib():
-    return _lib.load()
+    global _loaded
+    if _loaded is None:
+        _loaded = _lib.load()
+    return _loaded
 
 
 def _check(status: int):
@@ -52,24 +59,51 @@ def _dev(t: torch.Tensor, name: str, dtype=None, shape=None) -> int:
         raise TypeError(f"{name} must be a torch tensor")
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor (libexw runs on the GPU only)")
-    if t.device.index != torch.cuda.current_device():  # the kernels launch on the current device
+    if t.get_device() != torch.cuda.current_device():  # the kernels launch on the current device
         raise ValueError(f"{name} is on {t.device}, not on the current device cuda:{torch.cuda.current_device()} "
                          "(select it with torch.cuda.device)")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
     return t.data_ptr()
 
 
+# The handle of a device's current stream without a torch.cuda.Stream object around it (2 us of a small call); the
+# object where this torch does not have the function.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream, device) -> int:
     if stream is None:
+        if _raw_stream is not None and device.index is not None:
+            return _raw_stream(device.index)
         return torch.cuda.current_stream(device).cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+# Descriptor arrays for the C entry points that take them (read there, never written): packed as bytes, the pointers
+# computed from the base tensors (contiguous, so item f starts f strides on) instead of sliced out of them one by one.
+_FRAME = "PPPiii4x"
+assert struct.calcsize("@" + _FRAME) == ctypes.sizeof(_lib.ExwFrame)
+assert struct.calcsize("@PP") == ctypes.sizeof(_lib.ExwFrameOut)
+
+
+def _frames(color, depth, mv, F, W, H, cdt) -> bytes:
+    c, d, m, n = color.data_ptr(), depth.data_ptr(), mv.data_ptr(), W * H
+    cs = 3 * n * color.element_size()
+    return struct.pack("@" + _FRAME * F, *[v for f in range(F)
+                                           for v in (c + f * cs, d + 4 * n * f, m + 8 * n * f, W, H, cdt)])
+
+
+def _frame_outs(out, mask, count, W, H) -> bytes:
+    o, k, n = out.data_ptr(), mask.data_ptr(), W * H
+    os = 3 * n * out.element_size()
+    return struct.pack("@%dP" % (2 * count), *[v for q in range(count) for v in (o + q * os, k + q * n)])
 
 
 def _hw(depth: torch.Tensor):
@@ -103,9 +137,8 @@ def exw_motion_bounds(depth, mv, tile_bounds=None, frame_bounds=None, ws=None, s
         tile_bounds = torch.empty(((H + 7) // 8, (W + 7) // 8, 4), dtype=torch.float32, device=dev)
     if frame_bounds is None:
         frame_bounds = torch.empty(4, dtype=torch.float32, device=dev)
-    need = exw_workspace_bytes(OP_MOTION_BOUNDS, W, H)
     if ws is None:
-        ws = workspace(need, dev)
+        ws = workspace(exw_workspace_bytes(OP_MOTION_BOUNDS, W, H), dev)
     _check(lib().exw_motion_bounds(_dev(depth, "depth", torch.float32), _dev(mv, "mv", torch.float32, (2, H, W)),
                                    W, H, _dev(tile_bounds, "tile_bounds", torch.float32),
                                    _dev(frame_bounds, "frame_bounds", torch.float32), ws.data_ptr(), ws.numel(),
@@ -141,9 +174,8 @@ def exw_warp(color, depth, mv, keys, k: int, denom: int = 4, out=None, mask=None
 def exw_fill_holes(color, mask, ws=None, stream=None):
     """Stage (c), in place on ``color``.  Returns ``color``."""
     H, W = int(mask.shape[0]), int(mask.shape[1])
-    need = exw_workspace_bytes(OP_FILL_HOLES, W, H, _cdt(color))
     if ws is None:
-        ws = workspace(need, color.device)
+        ws = workspace(exw_workspace_bytes(OP_FILL_HOLES, W, H, _cdt(color)), color.device)
     _check(lib().exw_fill_holes(_dev(color, "color", None, (3, H, W)), _cdt(color),
                                 _dev(mask, "mask", torch.uint8, (H, W)), W, H, ws.data_ptr(), ws.numel(),
                                 _stream(stream, color.device)))
@@ -167,32 +199,25 @@ def exw_extrapolate(color, depth, mv, nfrac: int = 3, fill: bool = True, out=Non
     Returns (out [F][nfrac][3][H][W], mask [F][nfrac][H][W]) -- without the F axis for a single frame.
     ``tma=False`` sets EXW_FLAG_NO_TMA (global-memory source reads; identical results)."""
     single = color.dim() == 3
-    if single:
-        color, depth, mv = color.unsqueeze(0), depth.unsqueeze(0), mv.unsqueeze(0)
-    F, _, H, W = (int(s) for s in color.shape)
+    lead = () if single else (int(color.shape[0]),)
+    F = 1 if single else lead[0]
+    _, H, W = (int(v) for v in (color.shape if single else color.shape[1:]))
     dev = color.device
     cdt = _cdt(color)
     if out is None:
         out = torch.empty((F, nfrac, 3, H, W), dtype=color.dtype, device=dev)
     if mask is None:
         mask = torch.empty((F, nfrac, H, W), dtype=torch.uint8, device=dev)
-    _dev(color, "color", None, (F, 3, H, W))
-    _dev(depth, "depth", torch.float32, (F, H, W))
-    _dev(mv, "mv", torch.float32, (F, 2, H, W))
+    _dev(color, "color", None, lead + (3, H, W))
+    _dev(depth, "depth", torch.float32, lead + (H, W))
+    _dev(mv, "mv", torch.float32, lead + (2, H, W))
     _dev(out, "out", color.dtype, (F, nfrac, 3, H, W))
     _dev(mask, "mask", torch.uint8, (F, nfrac, H, W))
-    need = exw_workspace_bytes(OP_EXTRAPOLATE, W, H, cdt, F, nfrac)
     if ws is None:
-        ws = workspace(need, dev)
-    frames = (_lib.ExwFrame * F)()
-    outs = (_lib.ExwFrameOut * (F * nfrac))()
-    for f in range(F):
-        frames[f] = _lib.ExwFrame(color[f].data_ptr(), depth[f].data_ptr(), mv[f].data_ptr(), W, H, cdt)
-        for j in range(nfrac):
-            outs[f * nfrac + j] = _lib.ExwFrameOut(out[f, j].data_ptr(), mask[f, j].data_ptr())
+        ws = workspace(exw_workspace_bytes(OP_EXTRAPOLATE, W, H, cdt, F, nfrac), dev)
     flags = (0 if fill else FLAG_NO_FILL) | (0 if tma else FLAG_NO_TMA)
-    _check(lib().exw_extrapolate(ctypes.cast(frames, ctypes.c_void_p), F, int(nfrac), flags,
-                                 ctypes.cast(outs, ctypes.c_void_p), ws.data_ptr(), ws.numel(),
+    _check(lib().exw_extrapolate(_frames(color, depth, mv, F, W, H, cdt), F, int(nfrac), flags,
+                                 _frame_outs(out, mask, F * nfrac, W, H), ws.data_ptr(), ws.numel(),
                                  _stream(stream, dev)))
     if single:
         return out[0], mask[0]
@@ -233,22 +258,11 @@ def exw_extrapolate_host(color, depth, mv, nfrac: int = 3, fill: bool = True, ou
     need = exw_workspace_bytes(OP_EXTRAPOLATE, W, H, cdt, min(chunk, F) if chunk > 0 else min(8, F), nfrac)
     if ws is None:
         ws = workspace(need, dev)
-    fh = (_lib.ExwFrame * F)()
-    fd = (_lib.ExwFrame * F)()
-    oh = (_lib.ExwFrameOut * (F * nfrac))()
-    od = (_lib.ExwFrameOut * (F * nfrac))()
-    for f in range(F):
-        fh[f] = _lib.ExwFrame(color[f].data_ptr(), depth[f].data_ptr(), mv[f].data_ptr(), W, H, cdt)
-        fd[f] = _lib.ExwFrame(dc[f].data_ptr(), dd[f].data_ptr(), dm[f].data_ptr(), W, H, cdt)
-        for j in range(nfrac):
-            oh[f * nfrac + j] = _lib.ExwFrameOut(out[f, j].data_ptr(), mask[f, j].data_ptr())
-            od[f * nfrac + j] = _lib.ExwFrameOut(do[f, j].data_ptr(), dk[f, j].data_ptr())
     flags = (0 if fill else FLAG_NO_FILL) | (0 if tma else FLAG_NO_TMA)
-    _check(lib().exw_extrapolate_host(ctypes.cast(fh, ctypes.c_void_p), ctypes.cast(fd, ctypes.c_void_p), F,
-                                      int(nfrac), flags, ctypes.cast(oh, ctypes.c_void_p),
-                                      None if direct else ctypes.cast(od, ctypes.c_void_p), int(chunk),
-                                      ws.data_ptr(), ws.numel(),
-                                      _stream(stream, dev)))
+    _check(lib().exw_extrapolate_host(_frames(color, depth, mv, F, W, H, cdt), _frames(dc, dd, dm, F, W, H, cdt), F,
+                                      int(nfrac), flags, _frame_outs(out, mask, F * nfrac, W, H),
+                                      None if direct else _frame_outs(do, dk, F * nfrac, W, H), int(chunk),
+                                      ws.data_ptr(), ws.numel(), _stream(stream, dev)))
     return out, mask
 
 
@@ -289,12 +303,9 @@ def exw_warp_recursive(color, depth, mv, steps: int = 3, fill: bool = True, out=
     _dev(mask, "mask", torch.uint8, (steps, H, W))
     if ws is None:
         ws = workspace(exw_workspace_bytes(OP_WARP_RECURSIVE, W, H, _cdt(color)), dev)
-    outs = (_lib.ExwFrameOut * steps)()
-    for i in range(steps):
-        outs[i] = _lib.ExwFrameOut(out[i].data_ptr(), mask[i].data_ptr())
     _check(lib().exw_warp_recursive(_dev(color, "color", None, (3, H, W)), _cdt(color),
                                     _dev(depth, "depth", torch.float32), _dev(mv, "mv", torch.float32, (2, H, W)), W,
-                                    H, steps, 0 if fill else FLAG_NO_FILL, ctypes.cast(outs, ctypes.c_void_p),
+                                    H, steps, 0 if fill else FLAG_NO_FILL, _frame_outs(out, mask, steps, W, H),
                                     ws.data_ptr(), ws.numel(), _stream(stream, dev)))
     return [(out[i], mask[i]) for i in range(steps)]
 
@@ -380,26 +391,29 @@ def exw_tuner_report(tuner: int) -> str:
     return buf.value.decode()
 
 
-def _stream_descs(streams, outs, nfrac):
-    descs = (_lib.ExwStreamDesc * len(streams))()
-    for i, ((color, depth, mv), (out, mask)) in enumerate(zip(streams, outs)):
-        H, W = int(depth.shape[0]), int(depth.shape[1])
-        _dev(color, "color", None, (3, H, W))
-        _dev(depth, "depth", torch.float32, (H, W))
-        _dev(mv, "mv", torch.float32, (2, H, W))
-        _dev(out, "out", color.dtype, (nfrac, 3, H, W))
-        _dev(mask, "mask", torch.uint8, (nfrac, H, W))
-        descs[i].src = _lib.ExwFrame(color.data_ptr(), depth.data_ptr(), mv.data_ptr(), W, H, _cdt(color))
-        for j in range(nfrac):
-            descs[i].out[j] = _lib.ExwFrameOut(out[j].data_ptr(), mask[j].data_ptr())
-    return descs
+_STREAM = _FRAME + "6P"
+assert struct.calcsize("@" + _STREAM) == ctypes.sizeof(_lib.ExwStreamDesc)
+
+
+def _stream_descs(streams, outs, nfrac) -> bytes:
+    vals = []
+    for (color, depth, mv), (out, mask) in zip(streams, outs):
+        H, W = depth.shape
+        n, es = W * H, color.element_size()
+        vals += (_dev(color, "color", None, (3, H, W)), _dev(depth, "depth", torch.float32, (H, W)),
+                 _dev(mv, "mv", torch.float32, (2, H, W)), W, H, _cdt(color))
+        o, k = _dev(out, "out", color.dtype, (nfrac, 3, H, W)), _dev(mask, "mask", torch.uint8, (nfrac, H, W))
+        for j in range(MAX_FRAC):
+            vals += (o + 3 * n * es * j, k + n * j) if j < nfrac else (0, 0)
+    return struct.pack("@" + _STREAM * len(streams), *vals)
 
 
 def exw_batched_workspace_bytes(streams, nfrac: int = 3) -> int:
-    descs = (_lib.ExwStreamDesc * len(streams))()
-    for i, (color, depth, mv) in enumerate(streams):
-        descs[i].src = _lib.ExwFrame(0, 0, 0, int(depth.shape[1]), int(depth.shape[0]), _cdt(color))
-    return int(lib().exw_batched_workspace_bytes(ctypes.cast(descs, ctypes.c_void_p), len(streams), int(nfrac)))
+    vals = []
+    for color, depth, _ in streams:
+        vals += (0, 0, 0, int(depth.shape[1]), int(depth.shape[0]), _cdt(color), 0, 0, 0, 0, 0, 0)
+    return int(lib().exw_batched_workspace_bytes(struct.pack("@" + _STREAM * len(streams), *vals), len(streams),
+                                                 int(nfrac)))
 
 
 def exw_extrapolate_batched(streams, nfrac: int = 3, fill: bool = True, outs=None, ws=None, tuner=None, stream=None,
@@ -412,11 +426,10 @@ def exw_extrapolate_batched(streams, nfrac: int = 3, fill: bool = True, outs=Non
         outs = [(torch.empty((nfrac,) + tuple(c.shape), dtype=c.dtype, device=dev),
                  torch.empty((nfrac,) + tuple(d.shape), dtype=torch.uint8, device=dev)) for c, d, _ in streams]
     descs = _stream_descs(streams, outs, nfrac)
-    need = int(lib().exw_batched_workspace_bytes(ctypes.cast(descs, ctypes.c_void_p), len(streams), int(nfrac)))
     if ws is None:
-        ws = workspace(need, dev)
+        ws = workspace(int(lib().exw_batched_workspace_bytes(descs, len(streams), int(nfrac))), dev)
     flags = (0 if fill else FLAG_NO_FILL) | (0 if tma else FLAG_NO_TMA)
-    _check(lib().exw_extrapolate_batched(ctypes.cast(descs, ctypes.c_void_p), len(streams), int(nfrac), flags,
+    _check(lib().exw_extrapolate_batched(descs, len(streams), int(nfrac), flags,
                                          ws.data_ptr(), ws.numel(), tuner or None, _stream(stream, dev)))
     return outs
 
@@ -449,6 +462,10 @@ def exw_warp_backward(grad_out, color, depth, mv, keys, k: int, denom: int = 4, 
     return grad_color, grad_mv
 
 
+_TRAIN = _FRAME + "5P"
+assert struct.calcsize("@" + _TRAIN) == ctypes.sizeof(_lib.ExwTrainFrame)
+
+
 def exw_warp_l2_grad(color, depth, mv, targets, nfrac: int = 3, grad_color=None, grad_mv=None, loss=None, ws=None,
                      stream=None):
     """Forward warp, L2 loss and adjoint of P_1..P_nfrac for a batch of frames in one call (exw_warp_l2_grad):
@@ -479,15 +496,14 @@ def exw_warp_l2_grad(color, depth, mv, targets, nfrac: int = 3, grad_color=None,
     _dev(loss, "loss", torch.float64, (F,))
     if ws is None:
         ws = workspace(exw_workspace_bytes(OP_WARP_L2_GRAD, W, H, cdt, 1, nfrac), dev)
-    frames = (_lib.ExwTrainFrame * F)()
-    for f in range(F):
-        frames[f].src = _lib.ExwFrame(color[f].data_ptr(), depth[f].data_ptr(), mv[f].data_ptr(), W, H, cdt)
-        for j in range(nfrac):
-            frames[f].target[j] = targets[f, j].data_ptr()
-        frames[f].grad_color = grad_color[f].data_ptr()
-        frames[f].grad_mv = grad_mv[f].data_ptr()
-    _check(call(ctypes.cast(frames, ctypes.c_void_p), F, int(nfrac), loss.data_ptr(), ws.data_ptr(), ws.numel(),
-                _stream(stream, dev)))
+    c, d, m, t, n = color.data_ptr(), depth.data_ptr(), mv.data_ptr(), targets.data_ptr(), W * H
+    gc, gm, cs = grad_color.data_ptr(), grad_mv.data_ptr(), 3 * n * color.element_size()
+    frames = struct.pack("@" + _TRAIN * F, *[
+        v for f in range(F)
+        for v in (c + f * cs, d + 4 * n * f, m + 8 * n * f, W, H, cdt,
+                  *(t + cs * (f * nfrac + j) if j < nfrac else 0 for j in range(MAX_FRAC)), gc + 12 * n * f,
+                  gm + 8 * n * f)])
+    _check(call(frames, F, int(nfrac), loss.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream, dev)))
     return loss, grad_color, grad_mv
 
 
