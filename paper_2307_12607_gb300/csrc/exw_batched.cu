@@ -162,6 +162,7 @@ static bool build_params(EngineParams *ep, const EngineSpec *specs, int first, i
                 encode(fn, &ep->maps[i][2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, f.mv, f.W, f.H, 2, 4, bx, by);
             if (ok) st.stage = kStageTma;
         }
+        p.windows = st.stage != kStageNone ? 1 : 0;
         ep->loaders |= st.stage == kStageLoad ? 1 : 0;
         st.nregions = ceil_div(f.W, 32) * ceil_div(f.H, 32);
         st.ntiles = l.n5x * l.n5y;

@@ -135,6 +135,7 @@ struct alignas(16) TileParams {
     const uint64_t *keys;       // staged warp: global keys
     const uint8_t *mask_in;     // staged fill: input mask
     int W, H, nfrac, L, k0;     // fractions k0 .. k0 + nfrac - 1 of 2^L
+    int windows;                // engine: the tiles' source windows are staged (else every tile reads global memory)
     void *out_color[3];
     uint8_t *out_mask[3];
     const float4 *tile_bounds;

@@ -169,9 +169,10 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
             }
             unsigned m = __ballot_sync(0xFFFFFFFFu, reach);
             // Every region that can reach R carries the same one motion, and its sources are smooth: the plan is known
-            // without a look at the 8 x 8 tiles' landing rectangles (mode 5 uses neither those nor the candidates).
+            // without a look at the 8 x 8 tiles' landing rectangles (mode 5 uses neither those nor the candidates; a
+            // stream without windows splats every tile from its candidates).
             // (The 60-frame 1080p sequence 3681 -> 3669 us, a 4K frame 269.6 -> 268.0.)
-            if (m != 0u && nreg <= 32) {
+            if (m != 0u && nreg <= 32 && p.windows) {
                 const int first = __ffs(m) - 1;
                 const uint32_t ux = __shfl_sync(0xFFFFFFFFu, rmx, first), uy = __shfl_sync(0xFFFFFFFFu, rmy, first);
                 int wx0, wy0;
