@@ -32,8 +32,16 @@ __device__ __forceinline__ bool window_fits(Rect U) {
 // records the landing rectangle of every fraction, whether all candidate sources share one motion, and the
 // staging mode and window the fused kernel will use.
 // ------------------------------------------------------------------------------------------------------------
-template <typename CT, int WX, int WY>
-__device__ inline void plan_tile(const TileParams &p, int tile) {  // called by one whole warp
+// NW warps of a CTA (one tile per CTA, NW > 1) share the visits of the bounds tiles: warp wq takes every NW-th pass, and
+// their landing rectangles and motions meet in shared memory.
+template <int NW> struct PlanShare {
+    int r[NW][kMaxFrac][4];
+    uint32_t mx[NW], my[NW], flags[NW];  // flags: 1 some source reaches R, 2 not all of them carry (mx, my)
+    int ndesc;
+};
+template <> struct PlanShare<1> {};
+template <typename CT, int WX, int WY, int NW = 1>
+__device__ inline void plan_tile(const TileParams &p, int tile, PlanShare<NW> *sh = nullptr, int wq = 0) {  // NW whole warps
     const int lane = threadIdx.x & 31;
     const int X0 = (tile % p.n5x) * kFillTile, Y0 = (tile / p.n5x) * kFillTile;
     const int RX0 = X0 - 1, RY0 = Y0 - 1;
@@ -138,7 +146,11 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
     };
     // the candidates, compacted in visiting order into the plan's descriptors (none when there are too many)
     SplatTile *desc = p.pdesc != nullptr ? p.pdesc + (size_t)tile * kPlanDesc : nullptr;
-    int ndesc = 0;
+    int ndesc = 0, pass = 0;
+    if constexpr (NW > 1) {
+        if (threadIdx.x == 0) sh->ndesc = 0;
+        __syncthreads();
+    }
     // Two levels: the 32 x 32 regions within the frame-wide motion range whose bounds can reach R (one per lane),
     // then the 16 bounds tiles of each such region (two regions per pass, 16 lanes each).  A region's bounds
     // contain its tiles' bounds and the offsets are monotone in the motion, so no tile that reaches R is skipped.
@@ -178,7 +190,7 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
                 int wx0, wy0;
                 if (__all_sync(0xFFFFFFFFu, !reach || (one && rmx == ux && rmy == uy)) != 0 &&
                     uniform_window(ux, uy, wx0, wy0) && smooth_sources(ux, uy)) {
-                    if (lane == 0) {
+                    if (lane == 0 && wq == 0) {
                         TilePlan pl{};
                         pl.mode = 5;
                         pl.wx0 = wx0;
@@ -198,6 +210,7 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
                     l1 = __ffs(m) - 1;
                     m &= m - 1u;
                 }
+                if (NW > 1 && (pass++ % NW) != wq) continue;
                 const int src = lane < 16 ? l0 : l1;
                 const int qx = __shfl_sync(0xFFFFFFFFu, rxl, src < 0 ? 0 : src);
                 const int qy = __shfl_sync(0xFFFFFFFFu, ryl, src < 0 ? 0 : src);
@@ -207,6 +220,10 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
                     if (bx < p.nbx && by < p.nby) st = visit(bx, by);
                 }
                 const unsigned hm = __ballot_sync(0xFFFFFFFFu, st.fm != 0);
+                if constexpr (NW > 1) {
+                    if (lane == 0) ndesc = atomicAdd(&sh->ndesc, __popc(hm));
+                    ndesc = __shfl_sync(0xFFFFFFFFu, ndesc, 0);
+                }
                 const int slot = ndesc + __popc(hm & ((1u << lane) - 1u));
                 if (desc != nullptr && st.fm != 0 && slot < kPlanDesc) desc[slot] = st;
                 ndesc += __popc(hm);
@@ -230,7 +247,42 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
         mx = m0;
         my = m1;
     }
-    const bool smooth = uni && hasm && smooth_sources(mx, my);
+    bool any = hasm != 0u;
+    if constexpr (NW > 1) {
+        if (lane == 0) {
+#pragma unroll
+            for (int kk = 0; kk < kMaxFrac; ++kk)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sh->r[wq][kk][j] = r[kk][j];
+            sh->mx[wq] = mx;
+            sh->my[wq] = my;
+            sh->flags[wq] = (any ? 1u : 0u) | (uni ? 0u : 2u);
+        }
+        __syncthreads();
+        if (wq != 0) return;
+#pragma unroll
+        for (int q = 1; q < NW; ++q) {
+#pragma unroll
+            for (int kk = 0; kk < kMaxFrac; ++kk) {
+                r[kk][0] = min(r[kk][0], sh->r[q][kk][0]);
+                r[kk][1] = max(r[kk][1], sh->r[q][kk][1]);
+                r[kk][2] = min(r[kk][2], sh->r[q][kk][2]);
+                r[kk][3] = max(r[kk][3], sh->r[q][kk][3]);
+            }
+            const uint32_t f = sh->flags[q], qx = sh->mx[q], qy = sh->my[q];
+            uni = uni && !(f & 2u);
+            if (f & 1u) {
+                if (!any) {
+                    any = true;
+                    mx = qx;
+                    my = qy;
+                }
+                uni = uni && mx == qx && my == qy;
+            }
+        }
+        ndesc = sh->ndesc;
+    }
+    const bool smooth = uni && any && smooth_sources(mx, my);
     if (lane != 0) return;
     TilePlan pl{};
     Rect U{1 << 30, -(1 << 30), 1 << 30, -(1 << 30)};
@@ -255,7 +307,7 @@ __device__ inline void plan_tile(const TileParams &p, int tile) {  // called by 
     pl.ndesc = desc != nullptr && ndesc <= kPlanDesc ? ndesc : 0;
     if (U.empty()) {
         pl.mode = 4;
-    } else if (uni && hasm) {
+    } else if (uni && any) {
         int wx0, wy0;
         if (uniform_window(mx, my, wx0, wy0)) {
             pl.mode = smooth ? 5 : 0;
