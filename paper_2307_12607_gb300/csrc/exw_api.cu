@@ -452,10 +452,12 @@ exw_status exw_warp_recursive(const void *color, exw_dtype cdt, const float *dep
     const float *d = depth, *m = mv;
     cudaError_t e = cudaSuccess;
     const bool fill = (flags & EXW_FLAG_NO_FILL) == 0;
+    TileParams prev{};
+    static_assert(2 * sizeof(FrameHeader) <= kAlign, "the headers of two steps fit the section of one");
     for (int i = 0; i < steps && e == cudaSuccess; ++i) {
         // step i: warp the previous frame (the source for i = 0) by a quarter step of the motion it carries; one
         // kernel gathers, fills and carries (the depth and motion of the next step)
-        TileParams p = tile_params(fl, fws, W, H, 1, 2, 1, 0);
+        TileParams p = tile_params(fl, fws, W, H, 1, 2, 1, i & 1);  // two headers in turn
         p.color = c;
         p.depth = d;
         p.mv = m;
@@ -464,11 +466,16 @@ exw_status exw_warp_recursive(const void *color, exw_dtype cdt, const float *dep
         p.out_mask[0] = out[i].mask;
         const bool carry = i + 1 < steps;
         float *dn = carry ? (float *)(b + r.depth[i & 1]) : nullptr, *mn = carry ? (float *)(b + r.mv[i & 1]) : nullptr;
-        const size_t header = fill ? fl.headers + sizeof(FrameHeader) : 0;  // the fill's counters
-        e = launch_clear_keys(keys, (size_t)W * H, s, fws, header / 4);
-        if (e == cudaSuccess) e = launch_splat_global(d, m, W, H, 1, 2, keys, s);
+        if (i == 0 || !fill) {  // (with the first step's counters, the status word before them is zeroed)
+            e = launch_clear_keys(keys, (size_t)W * H, s, fws, fill ? (fl.headers + sizeof(FrameHeader)) / 4 : 0);
+            if (e == cudaSuccess) e = launch_splat_global(d, m, W, H, 1, 2, keys, s);
+        } else {  // the step before is finished on the way
+            e = launch_clear_coarse(prev, keys, (size_t)W * H, s, p.fh, sizeof(FrameHeader) / 4);
+            if (e == cudaSuccess) e = launch_splat_fixup(prev, cdt, d, m, W, H, 1, 2, keys, s);
+        }
         if (e == cudaSuccess) e = launch_warp(p, cdt, fill, dn, mn, s);
-        if (e == cudaSuccess && fill) e = launch_fixup(p, cdt, s);
+        if (e == cudaSuccess && fill && !carry) e = launch_fixup(p, cdt, s);
+        prev = p;
         d = dn;
         m = mn;
         c = out[i].color;

@@ -7,12 +7,10 @@ namespace exw {
 // zero_words words of a frame header to zero.  A block clears kClearPairs pairs, all of a thread's stores at immediate
 // offsets: 6.2 M keys took 41 instructions a store in a grid-stride loop.
 constexpr int kClearPerThread = 8, kClearPairs = 256 * kClearPerThread;
-__global__ void __launch_bounds__(256) clear_keys_kernel(unsigned long long *keys, uint32_t n, uint32_t *zero,
-                                                         uint32_t zero_words) {
-    grid_dependency_wait();
-    grid_dependents_launch();  // the splat
+__device__ __forceinline__ void clear_keys_block(unsigned long long *keys, uint32_t n, uint32_t block, uint32_t *zero,
+                                                 uint32_t zero_words) {
     const uint32_t head = ((uintptr_t)keys & 15u) ? 1u : 0u, npair = (n - head) / 2;
-    const uint32_t first = blockIdx.x * (uint32_t)kClearPairs + threadIdx.x;
+    const uint32_t first = block * (uint32_t)kClearPairs + threadIdx.x;
     ulonglong2 *pairs = reinterpret_cast<ulonglong2 *>(keys + head) + first;
     const ulonglong2 empty = make_ulonglong2(kKeyEmpty, kKeyEmpty);
     if (first + 256 * (kClearPerThread - 1) < npair) {
@@ -23,10 +21,28 @@ __global__ void __launch_bounds__(256) clear_keys_kernel(unsigned long long *key
         for (int u = 0; u < kClearPerThread; ++u)
             if (first + 256 * u < npair) pairs[256 * u] = empty;
     }
-    if (blockIdx.x != 0) return;
+    if (block != 0u) return;
     if (threadIdx.x == 0 && head) keys[0] = kKeyEmpty;
     if (threadIdx.x == 1 && head + 2 * npair < n) keys[n - 1] = kKeyEmpty;
     for (uint32_t i = threadIdx.x; i < zero_words; i += blockDim.x) zero[i] = 0u;
+}
+
+__global__ void __launch_bounds__(256) clear_keys_kernel(unsigned long long *keys, uint32_t n, uint32_t *zero,
+                                                         uint32_t zero_words) {
+    grid_dependency_wait();
+    grid_dependents_launch();  // the splat
+    clear_keys_block(keys, n, blockIdx.x, zero, zero_words);
+}
+
+// Between two steps of a recursive chain the last step's fill is finished by the kernels that clear and splat anyway,
+// which touch none of its data: here the first block runs the coarse pass of p, the others clear.  (Zeroed: the next
+// step's header, not p's.)
+__global__ void __launch_bounds__(256) clear_coarse_kernel(const __grid_constant__ TileParams p, unsigned long long *keys,
+                                                           uint32_t n, uint32_t *zero, uint32_t zero_words) {
+    grid_dependency_wait();  // the step's nodes; its reads of the keys
+    grid_dependents_launch();  // the splat
+    if (blockIdx.x == 0) coarse_pass(p);
+    else clear_keys_block(keys, n, blockIdx.x - 1, zero, zero_words);
 }
 
 __global__ void zero_kernel(uint32_t *p, size_t nwords) {
@@ -39,10 +55,8 @@ __global__ void zero_kernel(uint32_t *p, size_t nwords) {
 // Stage (a) into a global key buffer: kSplatRows source pixels of one column per thread, their loads issued together,
 // and a 64-bit atomicMin at each target (a warp's 32 targets of a row mostly share sectors).
 constexpr int kSplatRows = 4;
-__global__ void __launch_bounds__(256) splat_global_kernel(const float *__restrict__ depth,
-                                                           const float *__restrict__ mv, int W, int H, int k, int L,
-                                                           unsigned long long *keys) {
-    grid_dependency_wait();  // the keys are cleared by the kernel before
+__device__ __forceinline__ void splat_block(const float *__restrict__ depth, const float *__restrict__ mv, int W, int H,
+                                            int k, int L, unsigned long long *keys) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y0 = blockIdx.y * kSplatRows;
     if (x >= W) return;
     const float *mvy = mv + (size_t)W * H;
@@ -65,6 +79,25 @@ __global__ void __launch_bounds__(256) splat_global_kernel(const float *__restri
         atomicMin(keys + ((uint32_t)gy * (uint32_t)W + (uint32_t)gx),
                   (unsigned long long)pack_key_global(db[r], (uint32_t)y * (uint32_t)W + (uint32_t)x));
     }
+}
+
+__global__ void __launch_bounds__(256) splat_global_kernel(const float *__restrict__ depth,
+                                                           const float *__restrict__ mv, int W, int H, int k, int L,
+                                                           unsigned long long *keys) {
+    grid_dependency_wait();  // the keys are cleared by the kernel before
+    splat_block(depth, mv, W, H, k, L, keys);
+}
+
+// The same, and in the grid's rows from fix_row on the fix-up of the last step's tiles without a valid pixel.
+template <typename CT>
+__global__ void __launch_bounds__(256) splat_fixup_kernel(const __grid_constant__ TileParams p,
+                                                          const float *__restrict__ depth,
+                                                          const float *__restrict__ mv, int W, int H, int k, int L,
+                                                          unsigned long long *keys, uint32_t fix_row) {
+    grid_dependency_wait();  // the keys are cleared, the coarse values written
+    if (blockIdx.y < fix_row) splat_block(depth, mv, W, H, k, L, keys);
+    else fixup_slice<CT>(p, (blockIdx.y - fix_row) * gridDim.x + blockIdx.x, (gridDim.y - fix_row) * gridDim.x,
+                         (int)threadIdx.x, 256);
 }
 
 // Stage (a0): one 32 x 32 source region per CTA of 4 warps (8 rows each, 24 loads in flight per thread), up to 12
@@ -134,6 +167,33 @@ cudaError_t launch_clear_keys(uint64_t *keys, size_t n, cudaStream_t s, void *ze
     const cudaError_t e = launch_dependent(clear_keys_kernel, dim3(grid), dim3(256), 0, s, k, nk, z, nz);
     count_launch();
     timing_end("exw_clear_keys", s);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_clear_coarse(const TileParams &p, uint64_t *keys, size_t n, cudaStream_t s, void *zero,
+                                size_t zero_words) {
+    unsigned long long *const k = (unsigned long long *)keys;
+    uint32_t *const z = (uint32_t *)zero;
+    const uint32_t nk = (uint32_t)n, nz = (uint32_t)zero_words;
+    const unsigned grid = 1u + (unsigned)((n / 2 + kClearPairs) / kClearPairs);
+    timing_begin("exw_clear_coarse", s);
+    const cudaError_t e = launch_dependent(clear_coarse_kernel, dim3(grid), dim3(256), 0, s, p, k, nk, z, nz);
+    count_launch();
+    timing_end("exw_clear_coarse", s);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_splat_fixup(const TileParams &p, exw_dtype cdt, const float *depth, const float *mv, int W, int H,
+                               int k, int L, uint64_t *keys, cudaStream_t s) {
+    const unsigned gx = (unsigned)ceil_div(W, 256), gy = (unsigned)ceil_div(H, kSplatRows);
+    const dim3 g(gx, gy + (unsigned)ceil_div(304, (int)gx), 1);  // at least 304 blocks for the fix-up
+    unsigned long long *const kp = (unsigned long long *)keys;
+    timing_begin("exw_splat_fixup", s);
+    const cudaError_t e =
+        cdt == EXW_F32 ? launch_dependent(splat_fixup_kernel<float>, g, dim3(256), 0, s, p, depth, mv, W, H, k, L, kp, gy)
+                       : launch_dependent(splat_fixup_kernel<__half>, g, dim3(256), 0, s, p, depth, mv, W, H, k, L, kp, gy);
+    count_launch();
+    timing_end("exw_splat_fixup", s);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -38,7 +38,7 @@ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 // Per-frame bookkeeping, zeroed at the start of every call that uses it.
 struct FrameHeader {
     uint32_t acc[4];       // ordered-float maxima of -min mv_x, max mv_x, -min mv_y, max mv_y (0 = none)
-    uint32_t done;         // tiles finished (the CTA finishing the last one runs the coarse pyramid)
+    uint32_t done;         // batched path: (tile, fraction) items finished
     uint32_t ninvalid[3];  // fill tiles without any valid pixel, per fraction
     uint32_t cready;       // batched path: the coarse values of this frame are written
     uint32_t queue;        // next tile of the persistent kernel
@@ -181,6 +181,13 @@ cudaError_t launch_carry_motion(const uint64_t *keys, const uint8_t *mask, const
                                 int W, int H, float *depth_out, float *mv_out, cudaStream_t s);
 cudaError_t launch_splat_global(const float *depth, const float *mv, int W, int H, int k, int L, uint64_t *keys,
                                 cudaStream_t s);
+struct TileParams;
+// The coarse pass of p's fill and n keys cleared to empty (and zero_words words zeroed); the fix-up of p's tiles without a
+// valid pixel and a splat.
+cudaError_t launch_clear_coarse(const TileParams &p, uint64_t *keys, size_t n, cudaStream_t s, void *zero,
+                                size_t zero_words);
+cudaError_t launch_splat_fixup(const TileParams &p, exw_dtype cdt, const float *depth, const float *mv, int W, int H,
+                               int k, int L, uint64_t *keys, cudaStream_t s);
 cudaError_t launch_bounds(const float *depth, const float *mv, int W, int H, float4 *tile_bounds, float2 *tile_depth,
                           float4 *region_bounds, FrameHeader *fh, cudaStream_t s);
 cudaError_t launch_bounds_finalize(const FrameHeader *fh, float *frame_bounds, cudaStream_t s);

@@ -122,20 +122,6 @@ __device__ __forceinline__ void publish_node(const TileParams &p, float4 node, i
     }
 }
 
-// Count a finished tile; the CTA that finishes the last tile of the frame runs the coarse pass.  Only thread 0
-// wrote the tile's nodes and list entries, so only it needs the fence before counting.
-__device__ __forceinline__ void tile_done(const TileParams &p, int *last) {
-    if (threadIdx.x == 0) {
-        __threadfence();
-        *last = atomicAdd(&p.fh->done, 1u) == (uint32_t)(p.n5x * p.n5y) - 1u;
-    }
-    __syncthreads();
-    if (*last) {
-        __threadfence();
-        coarse_pass(p);
-    }
-}
-
 // ------------------------------------------------------------------------------------------------------------
 // Pull-push of one 32 x 32 tile by kTileThreads threads: lane = column, warp w the rows 2w and 2w + 1, so every row
 // access is one line and a thread's pixels need no index arithmetic of their own.  Level 1 of two columns' pixels is
