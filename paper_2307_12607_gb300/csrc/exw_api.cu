@@ -543,7 +543,7 @@ static exw_status warp_l2_grad(const exw_train_frame *frames, int nframes, int n
     if (entry_check() != EXW_OK) return EXW_ERR_CUDA;
     cudaError_t e = cudaSuccess;
     for (int f = 0; f < nframes && e == cudaSuccess; ++f)
-        e = launch_train_frame(frames[f], nfrac, loss + f, store, ws, (cudaStream_t)stream);
+        e = launch_train_frame(frames[f], f, nframes, nfrac, loss + f, store, ws, (cudaStream_t)stream);
     return from_cuda(e);
 }
 

@@ -3,30 +3,6 @@
 
 namespace exw {
 
-// n keys (8-byte aligned) to empty, in 16-byte stores (the first and last key alone where they do not pair up), and
-// zero_words words of a frame header to zero.  A block clears kClearPairs pairs, all of a thread's stores at immediate
-// offsets: 6.2 M keys took 41 instructions a store in a grid-stride loop.
-constexpr int kClearPerThread = 8, kClearPairs = 256 * kClearPerThread;
-__device__ __forceinline__ void clear_keys_block(unsigned long long *keys, uint32_t n, uint32_t block, uint32_t *zero,
-                                                 uint32_t zero_words) {
-    const uint32_t head = ((uintptr_t)keys & 15u) ? 1u : 0u, npair = (n - head) / 2;
-    const uint32_t first = block * (uint32_t)kClearPairs + threadIdx.x;
-    ulonglong2 *pairs = reinterpret_cast<ulonglong2 *>(keys + head) + first;
-    const ulonglong2 empty = make_ulonglong2(kKeyEmpty, kKeyEmpty);
-    if (first + 256 * (kClearPerThread - 1) < npair) {
-#pragma unroll
-        for (int u = 0; u < kClearPerThread; ++u) pairs[256 * u] = empty;
-    } else {
-#pragma unroll
-        for (int u = 0; u < kClearPerThread; ++u)
-            if (first + 256 * u < npair) pairs[256 * u] = empty;
-    }
-    if (block != 0u) return;
-    if (threadIdx.x == 0 && head) keys[0] = kKeyEmpty;
-    if (threadIdx.x == 1 && head + 2 * npair < n) keys[n - 1] = kKeyEmpty;
-    for (uint32_t i = threadIdx.x; i < zero_words; i += blockDim.x) zero[i] = 0u;
-}
-
 __global__ void __launch_bounds__(256) clear_keys_kernel(unsigned long long *keys, uint32_t n, uint32_t *zero,
                                                          uint32_t zero_words) {
     grid_dependency_wait();

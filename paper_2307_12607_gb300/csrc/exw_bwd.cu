@@ -19,8 +19,8 @@
 // Bound by issue.  The records are planes of words (each read without bank conflicts) with a mask of the directions a
 // winner's taps lie in, so phase 2 tests nine bits and reads four records a pixel instead of nine; element addresses are
 // 32-bit indices on per-plane pointers; the forward value is computed once for the loss and for the motion gradient.
-// 1080p FP32, three fractions: 201 us a frame before (674 instructions per output pixel), 155 us now (events around the
-// launch, 157 in a profile); splat 19 -> 15 us.
+// 1080p FP32, three fractions: 201 us a frame before (674 instructions per output pixel), 147 us now (events around the
+// launch); splat 19 -> 15 us.
 #include "exw_device.cuh"
 #include "exw_internal.h"
 
@@ -40,7 +40,6 @@ struct BwdSmem {
     uint16_t dirs[kRegionN];  // bit 3 (dy + 1) + dx + 1: the source pixel p + (dx, dy) is a tap of p (0: p won nothing)
     float depth[kStageN];   // NaN outside the frame (never lands, never agrees)
     double red[kBwdThreads / 32];
-    int last;
 };
 
 // Every plane by its own pointer, so that an element's address is one wide multiply-add of a 32-bit index (a plane has
@@ -56,8 +55,6 @@ struct BwdArgs {
     float *grad_mv[2];
     bool store;                      // the gradients are written (as if they were zero before), not accumulated
     double *partial;                 // fused: one loss partial per CTA
-    unsigned int *arrived;           // fused: CTAs finished (the last one sums the partials)
-    double *loss;                    // fused: the frame's loss
 };
 
 template <typename CT, bool FUSED>
@@ -269,37 +266,51 @@ __global__ void __launch_bounds__(kBwdThreads, 4) bwd_tile_kernel(const __grid_c
         a.grad_mv[1][i] = gm.y;
     }
     if constexpr (FUSED) {
-        // the loss: per CTA a fixed tree over its threads, then the CTAs in a fixed order by the last one to finish
+        // the loss: per CTA a fixed tree over its threads; the CTAs' partials are added by the next launch
         double lsum = (double)lacc;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, o);
         if (lane == 0) red[wid] = lsum;
         __syncthreads();
-        const unsigned int nblocks = gridDim.x * gridDim.y, bid = blockIdx.y * gridDim.x + blockIdx.x;
         if (tid == 0) {
             double t = 0.0;
             for (int w = 0; w < kBwdThreads / 32; ++w) t += red[w];
-            a.partial[bid] = t;
-            __threadfence();
-            sm.last = atomicAdd(a.arrived, 1u) == nblocks - 1u ? 1 : 0;
-        }
-        __syncthreads();
-        if (!sm.last) return;
-        __threadfence();
-        double t = 0.0;
-        for (unsigned int b = tid; b < nblocks; b += kBwdThreads) t += __ldcg(a.partial + b);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-        __syncthreads();
-        if (lane == 0) red[wid] = t;
-        __syncthreads();
-        if (tid == 0) {
-            double v = 0.0;
-            for (int w = 0; w < kBwdThreads / 32; ++w) v += red[w];
-            *a.loss = v;
-            *a.arrived = 0u;
+            a.partial[blockIdx.y * gridDim.x + blockIdx.x] = t;
         }
     }
+}
+
+// The loss of a frame from its CTAs' partials in a fixed order (one CTA, in a launch after the frame's: counted and summed
+// by the CTA that finished last, every CTA ended with a fence and an atomic's round trip -- eight frames of 1080p FP32
+// took 1318 us, now 1278).
+__device__ __forceinline__ void sum_loss(const double *partial, unsigned int n, double *loss) {
+    __shared__ double red[kBwdThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    double t = 0.0;
+    for (unsigned int b = tid; b < n; b += kBwdThreads) t += __ldcg(partial + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+    if (lane == 0) red[wid] = t;
+    __syncthreads();
+    if (tid == 0) {
+        double v = 0.0;
+        for (int w = 0; w < kBwdThreads / 32; ++w) v += red[w];
+        *loss = v;
+    }
+}
+__global__ void __launch_bounds__(kBwdThreads) loss_sum_kernel(const double *partial, unsigned int n, double *loss) {
+    grid_dependency_wait();  // the partials
+    sum_loss(partial, n, loss);
+}
+
+// Between two frames: the first block sums the last frame's loss, the others clear the keys for the next frame's splat.
+__global__ void __launch_bounds__(256) clear_loss_kernel(const double *partial, unsigned int npart, double *loss,
+                                                         unsigned long long *keys, uint32_t n) {
+    static_assert(kBwdThreads == 256, "the sum's threads");
+    grid_dependency_wait();  // the partials; the last frame's reads of the keys
+    grid_dependents_launch();  // the splat
+    if (blockIdx.x == 0) sum_loss(partial, npart, loss);
+    else clear_keys_block(keys, n, blockIdx.x - 1, nullptr, 0u);
 }
 
 // Stage (a) for fractions k0 .. k0 + nfrac - 1 in one pass: each source pixel is read once and takes the 64-bit
@@ -386,9 +397,9 @@ cudaError_t launch_backward(const float *grad_out, const void *color, exw_dtype 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Workspace of exw_warp_l2_grad: the key planes of the fractions, the CTAs' loss partials and the arrival counter.
+// Workspace of exw_warp_l2_grad: the key planes of the fractions and the CTAs' loss partials.
 struct TrainLayout {
-    size_t keys, partial, arrived, total;
+    size_t keys, partial, total;
 };
 static TrainLayout train_layout(int W, int H, int nfrac) {
     TrainLayout t{};
@@ -397,22 +408,33 @@ static TrainLayout train_layout(int W, int H, int nfrac) {
     off += align_up((size_t)nfrac * W * H * 8);
     t.partial = off;
     off += align_up((size_t)ceil_div(W, kFillTile) * ceil_div(H, kFillTile) * 8);
-    t.arrived = off;
-    off += kAlign;
-    t.total = off;
+    t.total = off + kAlign;  // (the last section is not used)
     return t;
 }
 
 size_t train_workspace_bytes(int W, int H, int nfrac) { return train_layout(W, H, nfrac).total; }
 
-// One frame of exw_warp_l2_grad: keys of every fraction (one clear, one splat pass), then the fused pass.
-cudaError_t launch_train_frame(const exw_train_frame &f, int nfrac, double *loss, bool store, void *ws,
-                               cudaStream_t s) {
+// Frame `frame` of nframes of exw_warp_l2_grad (loss: its loss): keys of every fraction (one clear, one splat pass), then
+// the fused pass.  A frame's loss is summed with the next frame's clear, the last one's by a launch of its own.
+cudaError_t launch_train_frame(const exw_train_frame &f, int frame, int nframes, int nfrac, double *loss, bool store,
+                               void *ws, cudaStream_t s) {
     const int W = f.src.W, H = f.src.H;
     const TrainLayout t = train_layout(W, H, nfrac);
     char *b = (char *)ws;
     unsigned long long *keys = (unsigned long long *)(b + t.keys);
-    cudaError_t e = launch_clear_keys((uint64_t *)keys, (size_t)nfrac * W * H, s, b + t.arrived, 1);
+    double *const partial = (double *)(b + t.partial);
+    const unsigned npart = (unsigned)(ceil_div(W, kFillTile) * ceil_div(H, kFillTile));
+    const size_t nkeys = (size_t)nfrac * W * H;
+    cudaError_t e;
+    if (frame == 0) {
+        e = launch_clear_keys((uint64_t *)keys, nkeys, s);
+    } else {
+        timing_begin("exw_clear_loss", s);
+        e = launch_dependent(clear_loss_kernel, dim3(1u + (unsigned)((nkeys / 2 + kClearPairs) / kClearPairs)), dim3(256), 0,
+                             s, (const double *)partial, npart, loss - 1, keys, (uint32_t)nkeys);
+        count_launch();
+        timing_end("exw_clear_loss", s);
+    }
     if (e != cudaSuccess) return e;
     timing_begin("exw_splat_multi", s);
     const int k0 = 1, L = 2;
@@ -434,14 +456,16 @@ cudaError_t launch_train_frame(const exw_train_frame &f, int nfrac, double *loss
     a.nfrac = nfrac;
     a.k0 = k0;
     a.L = L;
-    a.partial = (double *)(b + t.partial);
-    a.arrived = (unsigned int *)(b + t.arrived);
-    a.loss = loss;
+    a.partial = partial;
     a.store = store;
     timing_begin("exw_train", s);
     e = f.src.cdt == EXW_F32 ? launch_bwd_tiles<float, true>(a, s) : launch_bwd_tiles<__half, true>(a, s);
     count_launch();
     timing_end("exw_train", s);
+    if (e == cudaSuccess && frame + 1 == nframes) {
+        e = launch_dependent(loss_sum_kernel, dim3(1), dim3(kBwdThreads), 0, s, (const double *)partial, npart, loss);
+        count_launch();
+    }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -197,7 +197,7 @@ cudaError_t launch_plan(const TileParams &p, exw_dtype cdt, int shape, cudaStrea
 size_t recursive_workspace_bytes(int W, int H);
 size_t train_workspace_bytes(int W, int H, int nfrac);
 // store: the gradients are written instead of accumulated (here and in launch_backward).
-cudaError_t launch_train_frame(const exw_train_frame &f, int nfrac, double *loss, bool store, void *ws,
+cudaError_t launch_train_frame(const exw_train_frame &f, int frame, int nframes, int nfrac, double *loss, bool store, void *ws,
                                cudaStream_t s);
 
 // Frame statistics (exw_stats.cu): FP64 reductions into a small fixed workspace.
