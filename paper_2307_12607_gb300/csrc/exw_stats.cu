@@ -424,13 +424,16 @@ __global__ void __launch_bounds__(32) color_mse_sum_kernel(const double *part, d
 // columns of both images are loaded two rows ahead into registers and staged in the warp's own shared memory; each
 // lane filters its two columns horizontally from 12 neighbours and adds the result to the 11 outputs whose windows
 // hold the row, which stay in registers (a ring unrolled by 11 rows).  Nothing but the raw rows passes through shared
-// memory.  FP32 on values shifted by -1/2 (variances and covariance are shift-invariant; the shift keeps the raw
-// second moments small); only the sum of the two variances enters the index, so a^2 + b^2 is one map: four maps.
-// The per-position values are added as float pairs, FP64 per warp and beyond.
+// memory.  FP32, as the moments of s = (a - 1/2) + (b - 1/2) and d = a - b: with l the luminance term's and v the
+// variance term's denominator the index is (1 - D^2 / l) (1 - var d / v), so its distance from 1 is formed directly and
+// images that are alike lose nothing to cancellation.  The distances are added as float pairs, FP64 per warp and beyond.
+// The window's weights are rounded to multiples of 2^-26 with a sum of exactly 1 (a sum off by an ulp gives a flat bright
+// area a variance of its own).  Against FP64, frames half a pixel apart: 1e-9, where the moments of a and b gave 6e-8
+// (and 5e-8 with the kernel before, which filtered through shared memory).
 //
-// Bound by issue: per output 2 x 44 multiply-adds for the windows, 18 for the products, about 35 for the index.  1080p
-// FP32 136 us with the filtered maps in shared memory (a multiply-add per load, the sum on the FP64 pipe), 55 us now
-// (events around both launches).
+// Bound by issue: per output 2 x 44 multiply-adds for the windows, 12 for the squares, about 30 for the index.  1080p
+// FP32 136 us with the filtered maps in shared memory (a multiply-add per load, the sum on the FP64 pipe), 55 us from the
+// moments of a and b, 52.7 us now (events around both launches).
 constexpr int kSsimCols = 64, kSsimIn = kSsimCols + 10, kSsimPad = 80;
 constexpr int kSsimWarps = 4, kSsimThreads = 32 * kSsimWarps;
 constexpr int kSsimItems = 12 * 152;  // warps of one wave: 12 per SM of 152 at up to 168 registers
@@ -460,7 +463,7 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
     grid_dependents_launch();  // the kernel that adds the partials
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int OW = W - 10, OH = H - 10;
-    float g[6];  // the window's weights, symmetric: g[i] = weight i = weight 10 - i
+    float g[6];  // the window's weights, symmetric (g[i] = weight i = weight 10 - i), their sum exactly 1
     {
         float e[11], sum = 0.0f;
         for (int i = 0; i < 11; ++i) {
@@ -468,7 +471,8 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
             sum += e[i];
         }
 #pragma unroll
-        for (int i = 0; i < 6; ++i) g[i] = e[i] / sum;
+        for (int i = 0; i < 5; ++i) g[i] = rintf(e[i] / sum * 67108864.0f) * (1.0f / 67108864.0f);
+        g[5] = 1.0f - 2.0f * (((g[0] + g[1]) + (g[2] + g[3])) + g[4]);
     }
     const float C1 = 1e-4f, C2 = 9e-4f;
     double total = 0.0;
@@ -498,7 +502,7 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
             return v;
         };
         const bool ok0 = X0 + 2 * lane < OW, ok1 = X0 + 2 * lane + 1 < OW;
-        float acc[11][4][2];  // output row o in slot o mod 11: maps a, b, a^2 + b^2, ab of the lane's two columns
+        float acc[11][4][2];  // output row o in slot o mod 11: maps s, d, s^2, d^2 of the lane's two columns
         LinearSum sum;
         Row n0 = fetch(0), n1 = fetch(1);
         for (int base = 0; base < nrow; base += 11) {
@@ -510,26 +514,27 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
 #pragma unroll
                 for (int i = 0; i < 3; ++i) {
                     if (lane + 32 * i < kSsimPad) {
-                        st[0][lane + 32 * i] = to_f<CT>(n0.a[i]) - 0.5f;
-                        st[1][lane + 32 * i] = to_f<CT>(n0.b[i]) - 0.5f;
+                        const float x = to_f<CT>(n0.a[i]), y = to_f<CT>(n0.b[i]);
+                        st[0][lane + 32 * i] = (x - 0.5f) + (y - 0.5f);
+                        st[1][lane + 32 * i] = x - y;
                     }
                 }
                 n0 = n1;
                 n1 = fetch(r + 2);
                 __syncwarp();  // the row is staged (the other parity's reads ended before this row's writes began)
-                float va[12], vb[12], h[4][2];
+                float vs[12], vd[12], h[4][2];
 #pragma unroll
                 for (int j = 0; j < 6; ++j) {
                     const float2 x = *reinterpret_cast<const float2 *>(&st[0][2 * lane + 2 * j]);
                     const float2 y = *reinterpret_cast<const float2 *>(&st[1][2 * lane + 2 * j]);
-                    va[2 * j] = x.x;
-                    va[2 * j + 1] = x.y;
-                    vb[2 * j] = y.x;
-                    vb[2 * j + 1] = y.y;
+                    vs[2 * j] = x.x;
+                    vs[2 * j + 1] = x.y;
+                    vd[2 * j] = y.x;
+                    vd[2 * j + 1] = y.y;
                 }
 #pragma unroll
                 for (int j = 0; j < 12; ++j) {
-                    const float x = va[j], y = vb[j], q = fmaf(x, x, y * y), p = x * y;
+                    const float x = vs[j], y = vd[j], q = x * x, p = y * y;
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {  // column c takes neighbours c .. c + 10
                         const int i = j - c;
@@ -555,12 +560,12 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
                     const int slot = (u + 1) % 11;
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
-                        const float ma = acc[slot][0][c], mb = acc[slot][1][c];
-                        const float vab = acc[slot][2][c] - ma * ma - mb * mb, cab = acc[slot][3][c] - ma * mb;
-                        const float mua = ma + 0.5f, mub = mb + 0.5f;
-                        const float num = (2.0f * mua * mub + C1) * (2.0f * cab + C2);
-                        const float den = (mua * mua + mub * mub + C1) * (vab + C2);
-                        sum.add(c == 0 ? (ok0 ? num / den : 0.0f) : (ok1 ? num / den : 0.0f), 0.0f);
+                        const float ms = acc[slot][0][c], md = acc[slot][1][c];
+                        const float vs2 = fmaf(-ms, ms, acc[slot][2][c]), vd2 = fmaf(-md, md, acc[slot][3][c]);
+                        const float S = ms + 1.0f, D2 = md * md;
+                        const float l = fmaf(0.5f, fmaf(S, S, D2), C1), v = fmaf(0.5f, vs2 + vd2, C2);
+                        const float e = fmaf(D2, v - vd2, vd2 * l) / (l * v);
+                        sum.add((c == 0 ? ok0 : ok1) ? e : 0.0f, 0.0f);
                     }
                 }
             }
@@ -578,7 +583,7 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
 __global__ void __launch_bounds__(32) ssim_sum_kernel(const double *part, int nparts, double count, double *out) {
     grid_dependency_wait();  // the partials
     const double t = warp_sum(part, nparts);
-    if (threadIdx.x == 0) out[0] = t / count;
+    if (threadIdx.x == 0) out[0] = 1.0 - t / count;
 }
 
 }  // namespace
