@@ -68,9 +68,9 @@ def dist_env():
 # capture (a smaller launch; the engine's traffic grows in proportion to the frames of a launch), with the hash of
 # the kernel's sources (KERNEL_SOURCES) it was taken on: reported only while they are unchanged, else null.
 MEASURED_TRAFFIC = {
-    ("exw_engine", "sequence_1080p_fp32"): ((236.626e6 + 282.247e6) / 4, "1ffed5361dabe3d2"),
-    ("exw_engine", "warp_4k_fp16"): (105.047e6 + 130.172e6, "1ffed5361dabe3d2"),
-    ("exw_train", "fwd_bwd_1080p"): (215.129e6 + 28.325e6, "b1abf7c2171af943"),
+    ("exw_engine", "sequence_1080p_fp32"): ((236.325e6 + 280.781e6) / 4, "284a9619a0c282a8"),
+    ("exw_engine", "warp_4k_fp16"): (105.028e6 + 130.240e6, "284a9619a0c282a8"),
+    ("exw_train", "fwd_bwd_1080p"): (215.155e6 + 27.964e6, "1b83d9e846edf82d"),
 }
 
 

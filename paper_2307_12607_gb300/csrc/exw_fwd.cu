@@ -42,8 +42,8 @@ __global__ void __launch_bounds__(32 * kPlanShare) plan_shared_kernel(const __gr
 // round trips -- key, motion, taps -- are taken for a thread's rows together.
 //
 // Bound by issue and latency (about 350 instructions a pixel; DRAM at a fifth of its rate).  One recursive step at 1080p
-// FP32: gather, fill and carry 42 + 20 + 16 us as three kernels (keys through shared memory, a division per key), 42 us
-// as this one; the gather alone at 720p FP16 21 -> 16 us (events around each launch).
+// FP32: gather, fill and carry 42 + 20 + 16 us as three kernels (keys through shared memory, a division per key), 34 us
+// as this one; the gather alone at 720p FP16 21 -> 15 us (events around each launch).
 // ------------------------------------------------------------------------------------------------------------
 
 // Source index -> (x, y) without a division: inv = floor(2^32 / W) + 1 (saturated), so the quotient is at most one too
