@@ -10,6 +10,7 @@ Layouts (see include/exw.h): colour [3][H][W] float32/float16, depth [H][W] floa
 from __future__ import annotations
 
 import ctypes
+import math
 import struct
 
 import torch
@@ -104,6 +105,25 @@ def _frame_outs(out, mask, count, W, H) -> bytes:
     o, k, n = out.data_ptr(), mask.data_ptr(), W * H
     os = 3 * n * out.element_size()
     return struct.pack("@%dP" % (2 * count), *[v for q in range(count) for v in (o + q * os, k + q * n)])
+
+
+def _host_items(t, name, lead, item, size):
+    """Addresses of t[i] (t[i, j]) for every index below ``lead``, by the tensor's own shape: a contiguous host tensor
+    that may hold more than the call needs, but no fewer items, none shorter than ``item`` elements, and only elements
+    of ``size`` bytes -- the copies and the engine go by these addresses alone."""
+    n = len(lead)
+    if t.is_cuda or not t.is_contiguous():
+        raise ValueError(f"{name}: a contiguous host tensor is expected")
+    if t.element_size() != size:
+        raise TypeError(f"{name}: elements of {size} bytes are expected, got {t.dtype}")
+    if t.dim() < n or any(have < want for have, want in zip(t.shape, lead)) or math.prod(t.shape[n:]) < item:
+        raise ValueError(f"{name}: {' x '.join(map(str, lead))} items of {item} elements are expected, got shape "
+                         f"{tuple(t.shape)}")
+    at = [t.data_ptr()]
+    for d, count in enumerate(lead):
+        step = math.prod(t.shape[d + 1:]) * size
+        at = [a + i * step for a in at for i in range(count)]
+    return at
 
 
 def _hw(depth: torch.Tensor):
@@ -231,7 +251,8 @@ def exw_extrapolate_host(color, depth, mv, nfrac: int = 3, fill: bool = True, ou
     three streams inside the call.  Returns host (out [F][nfrac][3][H][W], mask [F][nfrac][H][W]) once the
     caller's stream has been synchronised.  dev_in = (colour, depth, motion) and dev_out = (out, mask): device
     staging tensors of the same shapes (allocated here when None).  direct=True: the engine writes the outputs
-    straight into the (page-locked) host tensors; dev_out is not used."""
+    straight into the (page-locked) host tensors; dev_out is not used.  Host tensors of the caller may be longer than the
+    call needs (more frames, fractions or planes): their own strides hold; shorter ones are refused."""
     F, _, H, W = (int(v) for v in color.shape)
     cdt = _cdt(color)
     dev = torch.device("cuda", torch.cuda.current_device())
@@ -239,9 +260,10 @@ def exw_extrapolate_host(color, depth, mv, nfrac: int = 3, fill: bool = True, ou
         out = torch.empty((F, nfrac, 3, H, W), dtype=color.dtype).pin_memory()
     if mask is None:
         mask = torch.empty((F, nfrac, H, W), dtype=torch.uint8).pin_memory()
-    for t, name in ((color, "color"), (depth, "depth"), (mv, "mv"), (out, "out"), (mask, "mask")):
-        if t.is_cuda or not t.is_contiguous():
-            raise ValueError(f"{name}: a contiguous host tensor is expected")
+    n, es = W * H, color.element_size()
+    sources = zip(_host_items(color, "color", (F,), 3 * n, es), _host_items(depth, "depth", (F,), n, 4),
+                  _host_items(mv, "mv", (F,), 2 * n, 4))
+    results = zip(_host_items(out, "out", (F, nfrac), 3 * n, es), _host_items(mask, "mask", (F, nfrac), n, 1))
     if dev_in is None:
         dev_in = (torch.empty_like(color, device=dev), torch.empty_like(depth, device=dev),
                   torch.empty_like(mv, device=dev))
@@ -259,8 +281,9 @@ def exw_extrapolate_host(color, depth, mv, nfrac: int = 3, fill: bool = True, ou
     if ws is None:
         ws = workspace(need, dev)
     flags = (0 if fill else FLAG_NO_FILL) | (0 if tma else FLAG_NO_TMA)
-    _check(lib().exw_extrapolate_host(_frames(color, depth, mv, F, W, H, cdt), _frames(dc, dd, dm, F, W, H, cdt), F,
-                                      int(nfrac), flags, _frame_outs(out, mask, F * nfrac, W, H),
+    frames = struct.pack("@" + _FRAME * F, *[v for src in sources for v in (*src, W, H, cdt)])
+    outs = struct.pack("@%dP" % (2 * F * nfrac), *[v for dst in results for v in dst])
+    _check(lib().exw_extrapolate_host(frames, _frames(dc, dd, dm, F, W, H, cdt), F, int(nfrac), flags, outs,
                                       None if direct else _frame_outs(do, dk, F * nfrac, W, H), int(chunk),
                                       ws.data_ptr(), ws.numel(), _stream(stream, dev)))
     return out, mask
