@@ -222,13 +222,13 @@ EXW_API exw_status exw_warp_recursive(const void *color, exw_dtype cdt, const fl
 /* Motion-variance features Var_x(F_mv), Var_y(F_mv) of the decision stage's environment vector E_t (Sec. IV-C,
  * Eq. 1; the feature is motivated in Sec. III-D): over every pixel of mv [2][H][W] whose two components are
  * finite, the population variance of the x component and of the y component.  out [3] is a DEVICE float64 array:
- * the number of pixels counted, Var_x, Var_y (0, 0 for an empty set).  FP64 throughout, merged in a fixed order:
- * deterministic.  Workspace: exw_workspace_bytes(EXW_OP_STATS, W, H, cdt, 1, 1). */
+ * the number of pixels counted, Var_x, Var_y (0, 0 for an empty set).  The sums have the accuracy of
+ * FP64 ones (error-free float words per thread, FP64 from a warp on) in a fixed order: deterministic.  Workspace: exw_workspace_bytes(EXW_OP_STATS, W, H, cdt, 1, 1). */
 EXW_API exw_status exw_mv_variance(const float *mv, int W, int H, double *out, void *ws, size_t ws_bytes,
                                    exw_stream_t stream);
 
-/* Mean squared difference of two colour images a, b [3][H][W] of type cdt over all 3 W H values (FP64, fixed
- * order): the MSE of the reward's PSNR = 10 log10(255^2 / MSE) (Sec. IV-C, Eq. 3) for colours in [0, 1] scaled by
+/* Mean squared difference of two colour images a, b [3][H][W] of type cdt over all 3 W H values (summed as in
+ * exw_mv_variance): the MSE of the reward's PSNR = 10 log10(255^2 / MSE) (Sec. IV-C, Eq. 3) for colours in [0, 1] scaled by
  * 255, i.e. PSNR = -10 log10(out[0]).  out [1] is a DEVICE float64.  Workspace: as exw_mv_variance. */
 EXW_API exw_status exw_color_mse(const void *a, const void *b, exw_dtype cdt, int W, int H, double *out, void *ws,
                                  size_t ws_bytes, exw_stream_t stream);

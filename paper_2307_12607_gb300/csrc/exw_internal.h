@@ -200,7 +200,7 @@ size_t train_workspace_bytes(int W, int H, int nfrac);
 cudaError_t launch_train_frame(const exw_train_frame &f, int frame, int nframes, int nfrac, double *loss, bool store, void *ws,
                                cudaStream_t s);
 
-// Frame statistics (exw_stats.cu): FP64 reductions into a small fixed workspace.
+// Frame statistics (exw_stats.cu): reductions of FP64 accuracy into a small fixed workspace.
 size_t stats_workspace_bytes();
 cudaError_t launch_mv_variance(const float *mv, int W, int H, double *out, void *ws, cudaStream_t s);
 cudaError_t launch_color_mse(const void *a, const void *b, exw_dtype cdt, int W, int H, double *out, void *ws,

@@ -3,11 +3,12 @@
 //
 // The sums keep FP64 accuracy without the FP64 pipe, which on this part takes one lane's operation per SM clock (a
 // warp instruction 32 clocks; the FP32 pipe takes 128 lanes): a thread forms each difference and square as a pair of
-// floats (two-difference, fused multiply-add residuals) and adds them with the error-free two-sum, the errors and the
-// small terms in words of their own; every kFoldValues values these are folded into a second set, so the small words
-// stay short sums.  Each rounding left is about 2^-48 of a short partial sum and independent of the others, so over an
-// image they average out below FP64's own last bit; short inputs, where they would not, and differences whose squares
-// would leave float's range go through FP64 value by value, as everything did before.
+// floats (two-difference, fused multiply-add residuals) and adds them error-free (two-sum) into words of falling size;
+// every kFoldValues values these are folded into a second set.  Short inputs, and differences whose squares would
+// leave float's range, go through FP64 value by value.  The error is at most that of
+// sums on the FP64 pipe, whether the values differ or repeat (the same operations in the same order on a host, 40
+// fields of each kind at 1080p and above, largest relative error: flat image pairs 2.4e-16 and 7.9e-15 in FP64, one
+// motion per object 2.5e-16 and 4.7e-16, stripes of four motions 1.2e-15 and 6.4e-15).
 //
 // Every grid is a function of the sizes only and every sum has a fixed order: results are deterministic and do not
 // depend on the GPU.  The blocks' partials are added by a one-block kernel launched behind them with programmatic
@@ -47,8 +48,8 @@ __device__ __forceinline__ float two_sum(float &s, float x) {  // s += x, return
     return e;
 }
 
-// A sum in words of falling size: s, the errors of its additions c, the rest d.  Adding values one by one leaves c and d
-// to plain additions (short sums); joining two sums is error-free down to d.
+// A sum in words of falling size: s, the errors of its additions c, the errors of c's additions d.  What is left to
+// plain additions is some 2^-72 of the sum.
 struct Words {
     float s = 0.0f, c = 0.0f, d = 0.0f;
     __device__ __forceinline__ void small(float x) { d = __fadd_rn(d, two_sum(c, x)); }
@@ -59,31 +60,44 @@ struct Words {
     }
 };
 
+// The words of a short sum hold one kind of term each, and every addition to them is error-free down to k: a plain
+// addition to any word but that rounds by up to 2^-48 of the sum, and where the values repeat -- one motion per object,
+// a flat image -- every thread rounds the same way, so that nothing averages out.
 struct LinearSum {  // of h + l: the short sum and the one it is folded into
     Words near, far;
+    float k = 0.0f;
     __device__ __forceinline__ void add(float h, float l) {
-        near.c = __fadd_rn(near.c, two_sum(near.s, h));
-        near.d = __fadd_rn(near.d, l);
+        k = __fadd_rn(k, two_sum(near.c, two_sum(near.s, h)));
+        k = __fadd_rn(k, two_sum(near.d, l));
     }
     __device__ __forceinline__ void fold() {
         far.small(near.d);
-        near.d = 0.0f;
+        near.d = k;
+        far.join(near);
+        near = Words{};
+        k = 0.0f;
+    }
+};
+
+struct FloatSum {  // of floats that are themselves rounded results: their sum to some 2^-48
+    Words near, far;
+    __device__ __forceinline__ void add(float x) { near.c = __fadd_rn(near.c, two_sum(near.s, x)); }
+    __device__ __forceinline__ void fold() {
         far.join(near);
         near = Words{};
     }
 };
 
-// Of (h + l)^2 = p + e + q + r + l^2 with p = fl(h h), q = fl(2 h l) and their exact residuals e, r.  Plain additions
-// of e would bias the sum by some 2^-51 of itself, so they are error-free too; each kind of term has a word of its own.
+// Of (h + l)^2 = p + e + q + r + l^2 with p = fl(h h), q = fl(2 h l) and their exact residuals e, r.
 struct SquareSum {
     Words near, far;
     float g = 0.0f, k = 0.0f;
     __device__ __forceinline__ void add(float h, float l) {
         const float p = __fmul_rn(h, h), h2 = 2.0f * h, q = __fmul_rn(h2, l);
         const float r = fmaf(l, l, fmaf(h2, l, -q));
-        near.c = __fadd_rn(near.c, two_sum(near.s, p));
+        k = __fadd_rn(k, two_sum(near.c, two_sum(near.s, p)));
         k = __fadd_rn(k, __fadd_rn(two_sum(near.d, fmaf(h, h, -p)), r));
-        g = __fadd_rn(g, q);
+        k = __fadd_rn(k, two_sum(g, q));
     }
     __device__ __forceinline__ void fold() {
         far.small(near.d);
@@ -503,7 +517,7 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
         };
         const bool ok0 = X0 + 2 * lane < OW, ok1 = X0 + 2 * lane + 1 < OW;
         float acc[11][4][2];  // output row o in slot o mod 11: maps s, d, s^2, d^2 of the lane's two columns
-        LinearSum sum;
+        FloatSum sum;
         Row n0 = fetch(0), n1 = fetch(1);
         for (int base = 0; base < nrow; base += 11) {
 #pragma unroll
@@ -565,7 +579,7 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
                         const float S = ms + 1.0f, D2 = md * md;
                         const float l = fmaf(0.5f, fmaf(S, S, D2), C1), v = fmaf(0.5f, vs2 + vd2, C2);
                         const float e = fmaf(D2, v - vd2, vd2 * l) / (l * v);
-                        sum.add((c == 0 ? ok0 : ok1) ? e : 0.0f, 0.0f);
+                        sum.add((c == 0 ? ok0 : ok1) ? e : 0.0f);
                     }
                 }
             }
