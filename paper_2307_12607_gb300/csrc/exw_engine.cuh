@@ -1100,20 +1100,32 @@ struct PendingCount {
 // alone, and its level-5 node matters only to the coarse pass of a fraction with a tile without any valid pixel -- which
 // most frames never run.  Such a tile publishes a placeholder instead of building its pyramid; when a coarse pass needs
 // the node (it lies under the first valid ancestor of an invalid tile), one warp computes it: a smooth tile from its
-// source colour (smooth_node), any other from its stored outputs and mask (output_node).
+// source colour (smooth_node), any other from its stored outputs and hole codes (output_node).
+//
+// The mask is an output only (a caller may give every fraction and stream the same plane), so which of the stored pixels
+// are holes has a place of its own: the tile's candidate list in the workspace, which nothing reads once the tile is
+// handed to the consumers.  A fraction takes a byte per thread of its group, two bits a pixel of the thread's block.
+// (Four ballots and a 16-byte store per warp instead: 4 frames of 1080p FP16 under a turning camera 392 us against 389, 48
+// streams 5085 and 5068.)
 constexpr float kNodeLazy = 2.0f;       // .w of a smooth tile's node that is not computed
 constexpr float kNodeNeeded = 3.0f;     // .w of a lazy smooth node the coarse pass needs
 constexpr float kNodeLazyOut = 4.0f;    // .w of the node of another such tile-fraction, not computed
 constexpr float kNodeNeededOut = 5.0f;  // .w of such a node the coarse pass needs
 
+static_assert(kMaxFrac * kGroupThreads <= kPlanDesc * (int)sizeof(SplatTile) && EXW_MASK_EMPTY < 4 && EXW_MASK_CRACK < 4,
+              "every fraction's hole codes fit the tile's candidate list");
+__device__ __forceinline__ uint8_t *hole_codes(const TileParams &p, int tile, int kk) {
+    return reinterpret_cast<uint8_t *>(p.pdesc + (size_t)tile * kPlanDesc) + kk * kGroupThreads;
+}
+
 // Fill and store one fraction of the tile for the calling group.  The group first votes on whether some hole has no valid
 // pixel in its 2 x 2 block (a barrier that also orders every read of the splat keys before their next initialisation).
 // Otherwise -- no hole, or scattered ones -- each thread fills its block from its own level-1 node and the group stores;
-// the tile publishes a lazy node, computed from what it stored only if a coarse pass needs it (the group's stores are
-// ordered before thread 0's count by a second barrier).  Else the pyramid is built: a second group barrier, at which a
-// warp without holes only arrives unless it is warp 0, which builds the upper levels.  c[] .w = validity.  (With the
-// pyramid for every tile-fraction with a hole, 4 frames of 1080p FP16 under a turning camera took 394, now
-// 387 us.)
+// the tile publishes a lazy node, computed from what it stored (the hole codes with it) only if a coarse pass needs it
+// (the group's stores are ordered before thread 0's count by a second barrier).  Else the pyramid is built: a second
+// group barrier, at which a warp without holes only arrives unless it is warp 0, which builds the upper levels.
+// c[] .w = validity.  (With the pyramid for every tile-fraction with a hole, 4 frames of 1080p FP16 under a turning camera
+// took 395, now 389 us; the 60-frame 1080p sequence 3690 and 3692.)
 template <typename CT>
 __device__ __forceinline__ void fill_store_block(EngineSmem &s, const TileParams &p, const FrameDims &d, CT *oc,
                                                  uint8_t *om, int g, int kk, int tile, int TX, int TY, float4 c[4],
@@ -1124,6 +1136,7 @@ __device__ __forceinline__ void fill_store_block(EngineSmem &s, const TileParams
     const bool all[4] = {true, true, true, true};
     const float4 n1 = mean4_01(c[0], c[1], c[2], c[3]);
     if (!bar_red_or(2 + g, kGroupThreads, hole && n1.w == 0.0f)) {
+        hole_codes(p, tile, kk)[tg] = (uint8_t)(m[0] + 4 * m[1] + 16 * m[2] + 64 * m[3]);
 #pragma unroll
         for (int t = 0; t < 4; ++t)
             if (m[t] != 0) c[t] = n1;
@@ -1217,8 +1230,8 @@ template <> __device__ __forceinline__ float load_out<__half>(const __half *q) {
     return __half2float(__ushort_as_half(__ldcg(reinterpret_cast<const unsigned short *>(q))));
 }
 
-// The level-5 node of a tile-fraction from its stored outputs and mask (one warp): the 2 x 2 blocks, the order and the
-// levels of fill_store_block, warp row w of the group as loop step w (a pixel outside the frame is invalid, as in the
+// The level-5 node of a tile-fraction from its stored outputs and hole codes (one warp): the 2 x 2 blocks, the order and
+// the levels of fill_store_block, warp row w of the group as loop step w (a pixel outside the frame is invalid, as in the
 // gather, and so is a hole, whatever it was filled with), so the same bits.
 template <typename CT>
 __device__ float4 output_node(const TileParams &p, int tile, int kk, float4 *l2) {
@@ -1226,7 +1239,7 @@ __device__ float4 output_node(const TileParams &p, int tile, int kk, float4 *l2)
     const int X0 = (tile % p.n5x) * kFillTile, Y0 = (tile / p.n5x) * kFillTile;
     const size_t plane = (size_t)p.W * p.H;
     const CT *oc = (const CT *)p.out_color[kk];
-    const uint8_t *om = p.out_mask[kk];
+    const uint8_t *codes = hole_codes(p, tile, kk);
 #pragma unroll 2
     for (int w = 0; w < kFillTile / 4; ++w) {
         const int TX = X0 + 2 * bx, TY = Y0 + 2 * (2 * w + (lane >> 4));
@@ -1239,7 +1252,7 @@ __device__ float4 output_node(const TileParams &p, int tile, int kk, float4 *l2)
                 const size_t q = (size_t)y * p.W + x;
                 const float4 v = make_float4(load_out<CT>(oc + q), load_out<CT>(oc + plane + q),
                                              load_out<CT>(oc + 2 * plane + q), 1.0f);
-                if (__ldcg(om + q) == 0) c[t] = v;
+                if (((__ldcg(codes + 32 * w + lane) >> (2 * t)) & 3u) == 0u) c[t] = v;
             }
         }
         const float4 n1 = mean4_01(c[0], c[1], c[2], c[3]);

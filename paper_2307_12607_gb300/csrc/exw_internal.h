@@ -142,7 +142,8 @@ struct alignas(16) TileParams {
     const float2 *tile_depth;   // per 8 x 8 tile: depth range of its pixels, (-1, -1) if one cannot land
     const float4 *region_bounds;  // per 32 x 32 region (fill tile): motion bounds of its 8 x 8 tiles
     TilePlan *plans;            // [n5] staging plan per target tile (persistent TMA kernel)
-    SplatTile *pdesc;           // [n5][kPlanDesc] candidate source tiles per target tile, or null
+    SplatTile *pdesc;           // [n5][kPlanDesc] candidate source tiles per target tile, or null; once a tile is taken,
+                                // its hole codes (the engine's fill)
     int nbx, nby;
     FrameHeader *fh;
     float4 *nodes;              // [nfrac][n5]
