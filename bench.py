@@ -76,8 +76,8 @@ MEASURED_TRAFFIC = {
 
 # The sources of each kernel and its host-side launch (the kernels whose traffic is recorded above).
 KERNEL_SOURCES = {
-    "exw_engine": ("exw_engine.cu", "exw_engine.cuh", "exw_items.cuh", "exw_tile.cuh", "exw_device.cuh",
-                   "exw_tma.cuh", "exw_internal.h", "exw_batched.cu"),
+    "exw_engine": ("exw_engine.cu", "exw_engine_kernel.cuh", "exw_engine.cuh", "exw_items.cuh", "exw_tile.cuh",
+                   "exw_device.cuh", "exw_tma.cuh", "exw_internal.h", "exw_batched.cu"),
     "exw_train": ("exw_bwd.cu", "exw_device.cuh", "exw_internal.h"),
 }
 ENGINE_SOURCES = KERNEL_SOURCES["exw_engine"]

@@ -1,5 +1,5 @@
 // exw_fwd.cu -- the staged kernels (exw_warp's gather, exw_fill_holes' fill) and the coarse fix-up; the fused
-// forward pass is the persistent engine (exw_engine.cu).
+// forward pass is the persistent engine (exw_engine.cuh).
 #include "exw_items.cuh"
 
 namespace exw {
