@@ -144,8 +144,8 @@ static bool build_params(EngineParams *ep, const EngineSpec *specs, int first, i
         p.status = ep->status;
         st.cdt = (int)f.cdt;
         // Windows by TMA where rows and bases are 16-byte aligned; else by the loader warps where every row starts at a
-        // whole word (all float colour, half colour of even width); else, or if the caller asked for it, global-memory
-        // reads.  1918 x 1079 FP32, 8 frames: global 1111 us, loaders 655; 1366 x 768 FP16: 548 and 382; 3838 x 2158
+        // whole word (all float colour, half colour of even width) and the launch has enough such tiles (below); else, or
+        // if the caller asked for it, global-memory reads.  1918 x 1079 FP32, 8 frames: global 1111 us, loaders 655; 1366 x 768 FP16: 548 and 382; 3838 x 2158
         // FP16 without fill: 462 and 270.  Half colour of odd width (1917 x 1079) would take 1255 against 1170: its
         // rows have to be shifted by half a word on the way.
         const int a = f.cdt == EXW_F16 ? 8 : 4;
@@ -162,11 +162,25 @@ static bool build_params(EngineParams *ep, const EngineSpec *specs, int first, i
                 encode(fn, &ep->maps[i][2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, f.mv, f.W, f.H, 2, 4, bx, by);
             if (ok) st.stage = kStageTma;
         }
-        p.windows = st.stage != kStageNone ? 1 : 0;
-        ep->loaders |= st.stage == kStageLoad ? 1 : 0;
         st.nregions = ceil_div(f.W, 32) * ceil_div(f.H, 32);
         st.ntiles = l.n5x * l.n5y;
         st.nfix = fill ? (int)kFixupItems : 0;
+    }
+    // The kernel with loader warps is some 3% slower for the streams that TMA stages, and a stream without windows costs
+    // its own tiles up to half more.  Loaders from 5% of a launch's tiles on: 47 streams of 4K FP16 with one of 854 x 480
+    // FP32 (0.1% of the tiles) take 9834 us with loaders and 9553 without; 24 of 1280 x 720 with one of 1278 x 720 (4.0%)
+    // 868 and 856; 16 of 1080p with one of 1918 x 1079 (5.9%) 1154 and 1176; 12 of 1080p FP16 with 4 of 1366 x 768 (14%)
+    // 1003 and 1046.
+    int tiles = 0, load_tiles = 0;
+    for (int i = 0; i < n; ++i) {
+        tiles += ep->st[i].ntiles;
+        if (ep->st[i].stage == kStageLoad) load_tiles += ep->st[i].ntiles;
+    }
+    ep->loaders = load_tiles > 0 && 20 * load_tiles >= tiles ? 1 : 0;
+    for (int i = 0; i < n; ++i) {
+        EngineStream &st = ep->st[i];
+        if (st.stage == kStageLoad && !ep->loaders) st.stage = kStageNone;
+        st.p.windows = st.stage != kStageNone ? 1 : 0;
     }
     // diagonal queue
     const int lag = sc.lag < 1 ? 1 : sc.lag;
