@@ -241,8 +241,10 @@ EXW_API exw_status exw_psnr(const void *a, const void *b, exw_dtype cdt, int W, 
 
 /* Structural similarity of two colour images a, b [3][H][W] of type cdt in [0, 1] (the SSIM of the reward, Sec.
  * IV-C, Eq. 3, read as the standard index: 11 x 11 Gaussian window, sigma 1.5, C1 = 1e-4, C2 = 9e-4, over every
- * window position wholly inside the image, averaged over positions and channels).  Moments in FP32 on values
- * shifted by -1/2, the mean in FP64 in a fixed order.  Needs W, H >= 11.  out [1] is a DEVICE float64.
+ * window position wholly inside the image, averaged over positions and channels).  Moments of the
+ * images' sum (less 1) and difference in FP32, each position's distance from 1 formed from them directly, its mean to
+ * FP64 accuracy in a fixed order: within some 1e-9 of the exact index where the images are alike or share nothing, 1e-6
+ * at worst (flat images of different brightness).  Needs W, H >= 11.  out [1] is a DEVICE float64.
  * Workspace: as exw_mv_variance. */
 EXW_API exw_status exw_ssim(const void *a, const void *b, exw_dtype cdt, int W, int H, double *out, void *ws,
                             size_t ws_bytes, exw_stream_t stream);

@@ -81,7 +81,9 @@ struct LinearSum {  // of h + l: the short sum and the one it is folded into
 
 struct FloatSum {  // of floats that are themselves rounded results: their sum to some 2^-48
     Words near, far;
-    __device__ __forceinline__ void add(float x) { near.c = __fadd_rn(near.c, two_sum(near.s, x)); }
+    __device__ __forceinline__ void add(float x, float low) {  // low: a correction smaller than x's last bit
+        near.c = __fadd_rn(near.c, __fadd_rn(two_sum(near.s, x), low));
+    }
     __device__ __forceinline__ void fold() {
         far.join(near);
         near = Words{};
@@ -198,8 +200,9 @@ template <typename CT, int N> __device__ __forceinline__ Pack<CT, N> load_pack(c
 constexpr int kShiftScan = 1024;
 
 // Partials: count, sums of x - kx and y - ky, sums of their squares, [5][kStatBlocks].  8 bytes read
-// and about 80 FP32 operations a pixel: 1080p 62 us with nine FP64 operations a pixel, 20.8 us now (events around
-// both launches; 2.4 us of reads at the copy rate, the rest launches, tails and issue).
+// and about 120 FP32 operations a pixel: 1080p 62 us with nine FP64 operations a pixel, 24 us now (events around
+// both launches; 2.4 us of reads at the copy rate, the rest launches, tails and issue; 22 with the errors of the words
+// added plainly, which biased repeated values).
 template <int N>
 __global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *__restrict__ mv, size_t n, bool wide,
                                                                    double *__restrict__ part) {
@@ -357,8 +360,8 @@ __global__ void __launch_bounds__(kSumThreads) mv_variance_sum_kernel(const doub
 // Colour MSE
 // ------------------------------------------------------------------------------------------------------------
 
-// 2c bytes read a pixel and about 30 FP32 operations a value: 1080p FP32 79 us with four FP64 operations a value,
-// 20.6 us now (events around both launches; 7.3 us of reads at the copy rate).
+// 2c bytes read a pixel and about 45 FP32 operations a value: 1080p FP32 79 us with four FP64 operations a value,
+// 22.5 us now (events around both launches; 7.3 us of reads at the copy rate).
 template <typename CT, int N>
 __global__ void __launch_bounds__(kStatThreads) color_mse_kernel(const CT *__restrict__ a, const CT *__restrict__ b,
                                                                  size_t n, bool wide, double *__restrict__ part) {
@@ -442,12 +445,14 @@ __global__ void __launch_bounds__(32) color_mse_sum_kernel(const double *part, d
 // variance term's denominator the index is (1 - D^2 / l) (1 - var d / v), so its distance from 1 is formed directly and
 // images that are alike lose nothing to cancellation.  The distances are added as float pairs, FP64 per warp and beyond.
 // The window's weights are rounded to multiples of 2^-26 with a sum of exactly 1 (a sum off by an ulp gives a flat bright
-// area a variance of its own).  Against FP64, frames half a pixel apart: 1e-9, where the moments of a and b gave 6e-8
-// (and 5e-8 with the kernel before, which filtered through shared memory).
+// area a variance of its own).  Error against FP64 over 12 pairs of 1280 x 720 each, rms, and that of a kernel which filtered
+// the moments of a and b through shared memory: smooth images half a pixel apart 5e-11 (2e-8), dark ones 3e-12 (3e-8),
+// inverted 3e-8 (3e-6), dark noise 2e-8 (1e-5), unrelated noise 2e-10 (8e-10), flat against noise 2e-9 (2e-9; at
+// 256 x 256 3e-9 and 2e-9).
 //
-// Bound by issue: per output 2 x 44 multiply-adds for the windows, 12 for the squares, about 30 for the index.  1080p
+// Bound by issue: per output 2 x 44 multiply-adds for the windows, 12 for the squares, about 36 for the index.  1080p
 // FP32 136 us with the filtered maps in shared memory (a multiply-add per load, the sum on the FP64 pipe), 55 us from the
-// moments of a and b, 52.7 us now (events around both launches).
+// moments of a and b, 53 us now (events around both launches).
 constexpr int kSsimCols = 64, kSsimIn = kSsimCols + 10, kSsimPad = 80;
 constexpr int kSsimWarps = 4, kSsimThreads = 32 * kSsimWarps;
 constexpr int kSsimItems = 12 * 152;  // warps of one wave: 12 per SM of 152 at up to 168 registers
@@ -577,9 +582,14 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
                         const float ms = acc[slot][0][c], md = acc[slot][1][c];
                         const float vs2 = fmaf(-ms, ms, acc[slot][2][c]), vd2 = fmaf(-md, md, acc[slot][3][c]);
                         const float S = ms + 1.0f, D2 = md * md;
-                        const float l = fmaf(0.5f, fmaf(S, S, D2), C1), v = fmaf(0.5f, vs2 + vd2, C2);
+                        const float l = fmaf(0.5f, fmaf(S, S, D2), C1);
+                        const float t = 0.5f * (vs2 + vd2), v = __fadd_rn(t, C2);
                         const float e = fmaf(D2, v - vd2, vd2 * l) / (l * v);
-                        sum.add((c == 0 ? ok0 : ok1) ? e : 0.0f);
+                        // v loses C2's low bits, the same ones wherever the variances have one magnitude: where the
+                        // images share nothing (e near 1) that alone moved the mean by 2e-9
+                        const float lost = __fsub_rn(C2, __fsub_rn(v, t)), low = -e * __fdividef(lost, v);
+                        const bool ok = c == 0 ? ok0 : ok1;
+                        sum.add(ok ? e : 0.0f, ok ? low : 0.0f);
                     }
                 }
             }
