@@ -120,8 +120,8 @@ __device__ __forceinline__ bool float_range(float h) {
 
 // d += x - y and q += (x - y)^2 in FP64 (not inlined: the FP64 instructions of the rare values stay off the others'
 // path).
-__device__ __noinline__ void wide_square(float x, float y, double &d, double &q) {
-    const double v = (double)x - (double)y;
+__device__ __noinline__ void wide_square(float x, double y, double &d, double &q) {
+    const double v = (double)x - y;
     d += v;
     q = fma(v, v, q);
 }
@@ -195,16 +195,80 @@ template <typename CT, int N> __device__ __forceinline__ Pack<CT, N> load_pack(c
 // Motion variance
 // ------------------------------------------------------------------------------------------------------------
 
+constexpr int kShiftScan = 1024;
+
 // Shift of the variance's sums: the first finite vector among the first kShiftScan pixels (0 when there is none);
 // every block finds the same one.  Any value of the field keeps the shifted sums' cancellation small.
-constexpr int kShiftScan = 1024;
+// By warp 0 of a block, into its shared memory (a block barrier comes before the others read it).
+__device__ __forceinline__ void find_shift(const float *__restrict__ mv, size_t n, float *shift) {
+    if (threadIdx.x >= 32) return;
+    int first = kShiftScan;
+    for (int i0 = 0; i0 < kShiftScan && (size_t)i0 < n && first == kShiftScan; i0 += 32) {
+        const int k = i0 + (int)threadIdx.x;
+        const float x = (size_t)k < n ? __ldg(mv + k) : __int_as_float(0x7FC00000);
+        const float y = (size_t)k < n ? __ldg(mv + n + k) : __int_as_float(0x7FC00000);
+        const unsigned int b = __ballot_sync(0xFFFFFFFFu, isfinite(x) && isfinite(y));
+        if (b) {
+            const int src = __ffs(b) - 1;
+            first = i0 + src;
+            const float sx = __shfl_sync(0xFFFFFFFFu, x, src), sy = __shfl_sync(0xFFFFFFFFu, y, src);
+            if (threadIdx.x == 0) {
+                shift[0] = sx;
+                shift[1] = sy;
+            }
+        }
+    }
+    if (threadIdx.x == 0 && first == kShiftScan) shift[0] = shift[1] = 0.0f;
+}
+
+// Inputs shorter than kWideValues: a vector per thread, FP64 throughout, over as many SMs as there are vectors for.  Both
+// launches at 64 x 64: 7.2 us; 22.1 through the FP64 path of the kernel below, which puts 2048 vectors on an SM (and 16.5
+// where all inputs were summed in FP64, 256 vectors a block).
+constexpr int kShortThreads = 128;
+static_assert((size_t)kStatBlocks * kShortThreads >= kWideValues, "a vector per thread");
+__global__ void __launch_bounds__(kShortThreads) mv_variance_short_kernel(const float *__restrict__ mv, size_t n,
+                                                                          double *__restrict__ part) {
+    constexpr int kWarps = kShortThreads / 32;
+    __shared__ float shift[2];
+    __shared__ double red[kWarps][5];
+    grid_dependency_wait();
+    grid_dependents_launch();  // the kernel that adds the partials
+    const size_t i = (size_t)blockIdx.x * kShortThreads + threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if ((size_t)blockIdx.x * kShortThreads >= n) {
+        if (threadIdx.x < 5) part[threadIdx.x * kStatBlocks + blockIdx.x] = 0.0;
+        return;
+    }
+    const float x = i < n ? __ldg(mv + i) : __int_as_float(0x7FC00000), y = i < n ? __ldg(mv + n + i) : x;
+    find_shift(mv, n, shift);
+    __syncthreads();
+    const bool ok = isfinite(x) && isfinite(y);
+    const double dx = ok ? (double)x - (double)shift[0] : 0.0, dy = ok ? (double)y - (double)shift[1] : 0.0;
+    double v[4] = {dx, dy, dx * dx, dy * dy};
+    const unsigned int count = __popc(__ballot_sync(0xFFFFFFFFu, ok));
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_xor_sync(0xFFFFFFFFu, v[c], o);
+    if (lane == 0) {
+        red[w][0] = (double)count;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) red[w][c + 1] = v[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < 5) {
+        double t = red[0][threadIdx.x];
+        for (int q = 1; q < kWarps; ++q) t += red[q][threadIdx.x];
+        part[threadIdx.x * kStatBlocks + blockIdx.x] = t;
+    }
+}
 
 // Partials: count, sums of x - kx and y - ky, sums of their squares, [5][kStatBlocks].  8 bytes read
 // and about 120 FP32 operations a pixel: 1080p 62 us with nine FP64 operations a pixel, 24 us now (events around
 // both launches; 2.4 us of reads at the copy rate, the rest launches, tails and issue; 22 with the errors of the words
 // added plainly, which biased repeated values).
 template <int N>
-__global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *__restrict__ mv, size_t n, bool wide,
+__global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *__restrict__ mv, size_t n,
                                                                    double *__restrict__ part) {
     __shared__ float shift[2];
     __shared__ Words shp[4][kStatWarps];
@@ -226,27 +290,10 @@ __global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *
         }
     };
     fetch(first_pack);  // the first values are on their way while the shift is found
-    if (threadIdx.x < 32) {
-        int first = kShiftScan;
-        for (int i0 = 0; i0 < kShiftScan && (size_t)i0 < n && first == kShiftScan; i0 += 32) {
-            const int k = i0 + (int)threadIdx.x;
-            const float x = (size_t)k < n ? __ldg(mv + k) : __int_as_float(0x7FC00000);
-            const float y = (size_t)k < n ? __ldg(mv + n + k) : __int_as_float(0x7FC00000);
-            const unsigned int b = __ballot_sync(0xFFFFFFFFu, isfinite(x) && isfinite(y));
-            if (b) {
-                const int src = __ffs(b) - 1;
-                first = i0 + src;
-                const float sx = __shfl_sync(0xFFFFFFFFu, x, src), sy = __shfl_sync(0xFFFFFFFFu, y, src);
-                if (threadIdx.x == 0) {
-                    shift[0] = sx;
-                    shift[1] = sy;
-                }
-            }
-        }
-        if (threadIdx.x == 0 && first == kShiftScan) shift[0] = shift[1] = 0.0f;
-    }
+    find_shift(mv, n, shift);
     __syncthreads();
     const float kx = shift[0], ky = shift[1];
+    const double kxd = (double)kx, kyd = (double)ky;  // converted once: a conversion costs as much as an FP64 addition
     unsigned int cnt = 0u;
     bool any_rare = false;
     LinearSum sx, sy;                       // sums of (x - kx), (y - ky)
@@ -259,7 +306,7 @@ __global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *
         float hx, lx, hy, ly;
         two_diff(x, kx, hx, lx);
         two_diff(y, ky, hy, ly);
-        const bool in = wide && float_range(hx) && float_range(hy), use = ok && in;
+        const bool in = float_range(hx) && float_range(hy), use = ok && in;
         hx = use ? hx : 0.0f;
         lx = use ? lx : 0.0f;
         hy = use ? hy : 0.0f;
@@ -271,8 +318,8 @@ __global__ void __launch_bounds__(kStatThreads) mv_variance_kernel(const float *
         return ok && !in;
     };
     auto take_rare = [&](float x, float y) {
-        wide_square(x, kx, r[0], r[2]);
-        wide_square(y, ky, r[1], r[3]);
+        wide_square(x, kxd, r[0], r[2]);
+        wide_square(y, kyd, r[1], r[3]);
     };
     static_assert(kFoldValues % (U * N) == 0, "whole rounds between folds");
     int round = 1;
@@ -408,14 +455,14 @@ __global__ void __launch_bounds__(kStatThreads) color_mse_kernel(const CT *__res
 #pragma unroll
                 for (int j = 0; j < N; ++j)
                     if (rare & (1u << (u * N + j)))
-                        wide_square(to_f<CT>(pa[u].v[j]), to_f<CT>(pb[u].v[j]), unused, r);
+                        wide_square(to_f<CT>(pa[u].v[j]), (double)to_f<CT>(pb[u].v[j]), unused, r);
         }
         if (round % (kFoldValues / (U * N)) == 0) q.fold();
     }
     const size_t tail = npack * N + first_pack;  // fewer than N values are left
     if (tail < n && take(a[tail], b[tail])) {
         any_rare = true;
-        wide_square(to_f<CT>(a[tail]), to_f<CT>(b[tail]), unused, r);
+        wide_square(to_f<CT>(a[tail]), (double)to_f<CT>(b[tail]), unused, r);
     }
     q.fold();
     double t = block_words(q.far, shp);
@@ -620,9 +667,11 @@ cudaError_t launch_mv_variance(const float *mv, int W, int H, double *out, void 
     const size_t n = (size_t)W * H;
     const bool vec = ((uintptr_t)mv & 15u) == 0 && (n & 3u) == 0;  // both planes start on 16 bytes
     timing_begin("exw_mv_variance", s);
-    const bool wide = n >= kWideValues;
-    cudaError_t e = launch_dependent(vec ? mv_variance_kernel<4> : mv_variance_kernel<1>, dim3(kStatBlocks),
-                                     dim3(kStatThreads), 0, s, mv, n, wide, part);
+    cudaError_t e =
+        n < kWideValues
+            ? launch_dependent(mv_variance_short_kernel, dim3(kStatBlocks), dim3(kShortThreads), 0, s, mv, n, part)
+            : launch_dependent(vec ? mv_variance_kernel<4> : mv_variance_kernel<1>, dim3(kStatBlocks),
+                               dim3(kStatThreads), 0, s, mv, n, part);
     count_launch();
     if (e == cudaSuccess) {
         const double *cpart = part;
