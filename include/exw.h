@@ -97,7 +97,8 @@ typedef enum exw_op {
 #define EXW_FLAG_NO_TMA 2u      /* read the source from global memory instead of staged shared-memory windows (identical
                                    results).  Windows are staged by TMA (16-byte aligned bases and W a multiple of 4
                                    for float32 colour, of 8 for float16 colour) or by copies of 4 or 8 bytes (any
-                                   float32 frame, float16 colour of even W on a 4-byte boundary), when possible */
+                                   float32 frame, float16 colour of even W on a 4-byte boundary), when possible; the
+                                   copies only where such frames hold 5% of the 32 x 32 tiles launched together */
 
 /* One source frame F_t (device pointers, layouts above). */
 typedef struct exw_frame {
@@ -111,7 +112,7 @@ typedef struct exw_frame {
 /* One extrapolated frame P_k (device pointers). */
 typedef struct exw_frame_out {
     void *color;    /* [3][H][W], same dtype as the source colour */
-    uint8_t *mask;  /* [H][W], EXW_MASK_* bits of stage (b) */
+    uint8_t *mask;  /* [H][W], EXW_MASK_* bits of stage (b); written, never read (planes of no use may coincide) */
 } exw_frame_out;
 
 /* Human-readable name of a status code (static storage). */

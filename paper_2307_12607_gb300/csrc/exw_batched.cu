@@ -145,9 +145,9 @@ static bool build_params(EngineParams *ep, const EngineSpec *specs, int first, i
         st.cdt = (int)f.cdt;
         // Windows by TMA where rows and bases are 16-byte aligned; else by the loader warps where every row starts at a
         // whole word (all float colour, half colour of even width) and the launch has enough such tiles (below); else, or
-        // if the caller asked for it, global-memory reads.  1918 x 1079 FP32, 8 frames: global 1111 us, loaders 655; 1366 x 768 FP16: 548 and 382; 3838 x 2158
-        // FP16 without fill: 462 and 270.  Half colour of odd width (1917 x 1079) would take 1255 against 1170: its
-        // rows have to be shifted by half a word on the way.
+        // if the caller asked for it, global-memory reads.  1918 x 1079 FP32, 8 frames: global 1111 us, loaders 655;
+        // 1366 x 768 FP16: 548 and 382; 3838 x 2158 FP16 without fill: 462 and 270.  Half colour of odd width (1917 x
+        // 1079) would take 1255 against 1170: its rows have to be shifted by half a word on the way.
         const int a = f.cdt == EXW_F16 ? 8 : 4;
         const bool words = f.cdt == EXW_F32 || ((f.W & 1) == 0 && ((uintptr_t)f.color & 3u) == 0);
         st.stage = sc.tma && words ? kStageLoad : kStageNone;

@@ -1,8 +1,10 @@
 // exw_device.cuh -- device-side building blocks of the warping fast path (sm_103a).
 //
-// Everything a kernel needs per pixel lives here so that the staged kernels (exw_splat_motion, exw_warp,
-// exw_fill_holes), the fused kernels and the batched kernel run literally the same arithmetic and agree bit for
-// bit.  Source data is read through an accessor (global memory or a shared-memory window staged by TMA).
+// What the staged kernels (exw_splat_motion, exw_warp, exw_fill_holes), the engine and the training pass compute per
+// pixel, so that they agree bit for bit: offsets, residuals, keys, the crack and tap rules, the weights' sum, roundings
+// and means.  The taps themselves are read and weighted in three places, each in its kernel's layout and all in the
+// same order: warp_kernel (exw_fwd.cu), gather_pixel (exw_engine.cuh), phase 1 of bwd_tile_kernel (exw_bwd.cu).  Source
+// data is read through an accessor (global memory or a staged shared-memory window).
 #pragma once
 
 #include <cstdint>

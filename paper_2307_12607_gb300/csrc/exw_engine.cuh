@@ -706,13 +706,6 @@ __device__ __forceinline__ void uniform_block(const Window<CT, WX, WY> &w, int w
     }
 }
 
-template <typename CT, int WX, int WY>
-__device__ __forceinline__ void uniform_block_any(const Window<CT, WX, WY> &w, int wx0, int wy0, const FrameDims &p,
-                                                  const UniformFrac &u, int TX, int TY, const uint32_t *words, int bx0,
-                                                  int by0, float4 c[4], uint8_t m[4]) {
-    uniform_block<CT, WX, WY>(w, wx0, wy0, p, u, TX, TY, words, bx0, by0, c, m);
-}
-
 // ------------------------------------------------------------------------------------------------------------
 // Tiles through splat keys (modes 1-3)
 // ------------------------------------------------------------------------------------------------------------
@@ -1221,9 +1214,7 @@ __device__ __forceinline__ float4 smooth_level2(const CT out[4][3]) {
     return right ? mean4_01(Ap, A, Bp, B) : mean4_01(A, Ap, B, Bp);
 }
 
-// The lazy smooth node, recomputed by one warp: the tile's outputs again from the source colour (the same arithmetic
-// as smooth_column_t, so the same bits), then the same pyramid.
-
+// A stored output pixel, as another CTA may have written it.
 template <typename CT> __device__ __forceinline__ float load_out(const CT *q);
 template <> __device__ __forceinline__ float load_out<float>(const float *q) { return __ldcg(q); }
 template <> __device__ __forceinline__ float load_out<__half>(const __half *q) {
@@ -1267,6 +1258,8 @@ __device__ float4 output_node(const TileParams &p, int tile, int kk, float4 *l2)
     return l5;
 }
 
+// The lazy smooth node, recomputed by one warp: the tile's outputs again from the source colour (the same arithmetic as
+// smooth_column_t, so the same bits), then the same pyramid.
 template <typename CT>
 __device__ float4 smooth_node(const TileParams &p, int tile, int kk, float4 *l2) {
     const int lane = threadIdx.x & 31;
@@ -1572,7 +1565,7 @@ __device__ __forceinline__ void tile_group(EngineSmem &s, const TileSlot &sl, co
         group_source_words(win, wx0, wy0, d, words, bx0, by0, __uint_as_float(sl.plan.umx),
                            __uint_as_float(sl.plan.umy), tg);
         bar_sync(kBarBounds + g, kGroupThreads);  // every word before any read of them
-        uniform_block_any<CT, WX, WY>(win, wx0, wy0, d, u, TX, TY, words, bx0, by0, c, m);
+        uniform_block<CT, WX, WY>(win, wx0, wy0, d, u, TX, TY, words, bx0, by0, c, m);
     } else if (mode == 1) {
         const WinAcc<CT, WX, WY> wa{&win, wx0, wy0};
         gather_block<CT>(key[kk], wa, d, k, TX, TY, bx, by, c, m);

@@ -1,6 +1,5 @@
-// exw_items.cuh -- the work items of the forward pass as device functions of a whole CTA (or warp): a bounds
-// region, a tile plan, a fused tile (TMA windows or global memory), a fix-up slice.  The per-frame kernels launch
-// them one item per CTA or in a persistent loop; the batched kernel takes them from a work queue.
+// exw_items.cuh -- the work items of the forward pass that kernels of their own and the persistent engine share: a bounds
+// region (four warps), a tile plan (one warp, or four of a small frame's plan kernel), a slice of the fix-up.
 #pragma once
 
 #include "exw_tile.cuh"
