@@ -81,8 +81,8 @@ struct LinearSum {  // of h + l: the short sum and the one it is folded into
 
 struct FloatSum {  // of floats that are themselves rounded results: their sum to some 2^-48
     Words near, far;
-    __device__ __forceinline__ void add(float x, float low) {  // low: a correction smaller than x's last bit
-        near.c = __fadd_rn(near.c, __fadd_rn(two_sum(near.s, x), low));
+    __device__ __forceinline__ void add(float x, float f) {  // x - f x, f x being smaller than x's last bit
+        near.c = __fadd_rn(near.c, fmaf(-f, x, two_sum(near.s, x)));
     }
     __device__ __forceinline__ void fold() {
         far.join(near);
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(32) color_mse_sum_kernel(const double *part, d
 // inverted 3e-8 (3e-6), dark noise 2e-8 (1e-5), unrelated noise 2e-10 (8e-10), flat against noise 2e-9 (2e-9; at
 // 256 x 256 3e-9 and 2e-9).
 //
-// Bound by issue: per output 2 x 44 multiply-adds for the windows, 12 for the squares, about 36 for the index.  1080p
+// Bound by issue: per output 2 x 44 multiply-adds for the windows, 12 for the squares, about 34 for the index.  1080p
 // FP32 136 us with the filtered maps in shared memory (a multiply-add per load, the sum on the FP64 pipe), 55 us from the
 // moments of a and b, 53 us now (events around both launches).
 constexpr int kSsimCols = 64, kSsimIn = kSsimCols + 10, kSsimPad = 80;
@@ -634,9 +634,8 @@ __global__ void __launch_bounds__(kSsimThreads, 3) ssim_kernel(const CT *__restr
                         const float e = fmaf(D2, v - vd2, vd2 * l) / (l * v);
                         // v loses C2's low bits, the same ones wherever the variances have one magnitude: where the
                         // images share nothing (e near 1) that alone moved the mean by 2e-9
-                        const float lost = __fsub_rn(C2, __fsub_rn(v, t)), low = -e * __fdividef(lost, v);
-                        const bool ok = c == 0 ? ok0 : ok1;
-                        sum.add(ok ? e : 0.0f, ok ? low : 0.0f);
+                        const float lost = __fsub_rn(C2, __fsub_rn(v, t));
+                        sum.add((c == 0 ? ok0 : ok1) ? e : 0.0f, __fdividef(lost, v));
                     }
                 }
             }
