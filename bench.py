@@ -68,9 +68,9 @@ def dist_env():
 # capture (a smaller launch; the engine's traffic grows in proportion to the frames of a launch), with the hash of
 # the kernel's sources (KERNEL_SOURCES) it was taken on: reported only while they are unchanged, else null.
 MEASURED_TRAFFIC = {
-    ("exw_engine", "sequence_1080p_fp32"): ((236.325e6 + 280.781e6) / 4, "284a9619a0c282a8"),
-    ("exw_engine", "warp_4k_fp16"): (105.028e6 + 130.240e6, "284a9619a0c282a8"),
-    ("exw_train", "fwd_bwd_1080p"): (215.155e6 + 27.964e6, "1b83d9e846edf82d"),
+    ("exw_engine", "sequence_1080p_fp32"): ((236.337e6 + 282.697e6) / 4, "f8ea5e394db63909"),
+    ("exw_engine", "warp_4k_fp16"): (105.012e6 + 130.267e6, "f8ea5e394db63909"),
+    ("exw_train", "fwd_bwd_1080p"): (215.155e6 + 27.637e6, "2950c214015f1091"),
 }
 
 
